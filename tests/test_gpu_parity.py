@@ -295,6 +295,20 @@ def test_logdet_slq_matches_oracle_with_identical_probes(gp, ctx, precond):
     assert abs(info["logdet"] - e["logdet"]) <= 5 * info["logdet_stderr"] + 1e-9 * abs(e["logdet"])
 
 
+@pytest.mark.parametrize("steps,rel", [(1, 1e-9), (2, 1e-9), (33, 1e-9), (257, 1e-6), (300, 1e-6)])
+def test_slq_quadrature_matches_the_oracle_eigensolve(gp, ctx, steps, rel):
+    """The quadrature of log T without its eigen-decomposition against the oracle's Gauss quadrature, in
+    FP64 with identical probes: one and two steps, a few tens, and more rows of T than the CTA has
+    threads.  Up to 33 steps T agrees to rounding (1e-13 per entry, times T's condition number of
+    at most 1e4); beyond that the two Lanczos processes lose orthogonality at different steps."""
+    import oracle
+    w = W.random_small(303, 3000, 2, L=3, sigma2=1e-2)
+    opts = gp.default_opts(precision=gp.PREC_FP64, logdet=gp.LOGDET_SLQ, probes=16, lanczos_steps=steps, seed=4)
+    _, info = ctx.lml(w["X"], w["y"], gp.Hyper(**w["hyper"]), opts)
+    s = oracle.lml_slq(w["X"], w["y"], oracle.Hyper(**w["hyper"]), m=16, k=steps, seed=4, grad=False)
+    assert info["logdet"] == pytest.approx(s["logdet"], rel=rel)
+
+
 @pytest.mark.parametrize("precond", [1, 2])
 def test_gradient_matches_oracle_hutchinson(gp, ctx, precond):
     import oracle
