@@ -397,7 +397,7 @@ gp2s_status gp2s_mcmc(gp2s_ctx *ctx, int64_t n, const double *X, const double *y
  * It computes what gp2s_lml computes with GP2S_PREC_FP64 and GP2S_LOGDET_EXACT, for n <=
  * GP2S_NOALLOC_MAX_N points: the dense FP64 matrix A = K + sigma2 I (same exact support test and
  * kernel as the CSR path), its Cholesky factor, log|A|, a = A^{-1} y, and the LML.  All scratch
- * lives in one fixed-size array compiled into the library (about 2.1 MB of every GPU that loads the
+ * lives in one fixed-size array compiled into the library (about 1.3 MB of every GPU that loads the
  * library, held until the process exits); the call makes no cudaMalloc / cudaFree and calls no
  * allocating library routine.
  *   n: 1..GP2S_NOALLOC_MAX_N; larger n returns GP2S_EINVAL and does nothing.

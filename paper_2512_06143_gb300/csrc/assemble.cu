@@ -878,6 +878,7 @@ gp2s_status assemble_problem(gp2s_ctx *c, int64_t n, const double *X_dev, const 
         return refresh_values(c, h, o);
     c->pat_valid = false;
     c->rb_pattern_valid = false;
+    c->chol_plan_valid = false;
     cudaEvent_t ev[5];
     for (int k = 0; k < 5; ++k) GP2S_CUDA(c, cudaEventCreate(&ev[k]));
     struct EvGuard { cudaEvent_t *e; ~EvGuard() { for (int k = 0; k < 5; ++k) cudaEventDestroy(e[k]); } } guard{ev};

@@ -210,7 +210,7 @@ static gp2s_status do_solve(gp2s_ctx *c, int method, int m, CGResult *res)
     const Assembled &A = c->A;
     if (method == GP2S_LOGDET_EXACT && m == 0 && A.opts.solver == GP2S_SOLVER_CG) {
         double ld = 0.0;
-        GP2S_TRY(exact_logdet_solve(c, c->ys64.as<double>(), &ld, false));
+        GP2S_TRY(exact_logdet_solve(c, c->ys64.as<double>(), &ld));
         double rr = 0.0;
         GP2S_TRY(y_residual(c, c->ys64.as<double>(), &rr));
         res->relres = rr;
@@ -310,7 +310,7 @@ void gp2s_destroy(gp2s_ctx *c)
                       &c->scan_tmp, &c->scan_tmp2, &c->cell_start, &c->cell_flag, &c->items, &c->item_cnt,
                       &c->B64, &c->B32, &c->D64, &c->s64, &c->s32, &c->rowcnt, &c->rowptr, &c->col,
                       &c->val32, &c->val64, &c->counters, &c->vec, &c->vec64, &c->partials, &c->scal,
-                      &c->Z, &c->Zf, &c->rec, &c->rsplit, &c->dense, &c->H, &c->gpart,
+                      &c->Z, &c->Zf, &c->rec, &c->rsplit, &c->dense, &c->chol_ints, &c->H, &c->gpart,
                       &c->rb_cnt, &c->rb_ptr, &c->rb_col, &c->rb_val, &c->rb_tpart, &c->rb_seg,
                       &c->bj_Minv, &c->bj_ld, &c->bj_Minv_y, &c->post_X, &c->post_B, &c->post_cnt,
                       &c->post_part, &c->mr_vec, &c->mc_X, &c->mc_y, &c->wc_lam, &c->wc_sig, &c->ff_mask,
@@ -412,7 +412,7 @@ gp2s_status gp2s_logdet(gp2s_ctx *c, double *logdet, double *stderr_hat, gp2s_lo
     double ldiag = 0.0, lhat = 0.0, se = 0.0;
     GP2S_TRY(sum_log_diag(c, &ldiag));
     if (method == GP2S_LOGDET_EXACT) {
-        GP2S_TRY(exact_logdet_solve(c, nullptr, &lhat, false));
+        GP2S_TRY(exact_logdet_solve(c, nullptr, &lhat));
     } else {
         const int m = A.opts.probes;
         if (m <= 0) return set_err(c, GP2S_EINVAL, "SLQ needs probes > 0");
@@ -476,7 +476,7 @@ static gp2s_status lml_impl(gp2s_ctx *c, int64_t n, const double *X, const doubl
     GP2S_TRY(sum_log_diag(c, &ldiag));
     if (method == GP2S_LOGDET_EXACT) {
         if (c->have_exact) lhat = c->exact_lhat;      // factored by the dense solve
-        else GP2S_TRY(exact_logdet_solve(c, nullptr, &lhat, false));
+        else GP2S_TRY(exact_logdet_solve(c, nullptr, &lhat));
     } else {
         GP2S_TRY(slq_logdet(c, m, o->lanczos_steps, &lhat, &se));
     }

@@ -154,8 +154,11 @@ struct gp2s_ctx {
     };
     std::map<int, TuneState> tune;
     std::mutex tune_mu;
-    // dense
-    gp2s::DevBuf dense;
+    // exact log-determinant: the factor's tiles, flags and solve vectors, and the pattern's plan (task list
+    // and tile structure) with its sizes
+    gp2s::DevBuf dense, chol_ints;
+    bool chol_plan_valid = false;   // chol_ints belongs to the current pattern
+    int chol_nt = 0, chol_ntiles = 0, chol_ntasks = 0;
     // adjoint
     gp2s::DevBuf H, gpart;
     // posterior (test points, their bump values / prior variances / outputs, counters, partials)
@@ -181,7 +184,7 @@ struct gp2s_ctx {
     int32_t solve_iters = 0, solve_outer = 0;
     double solve_relres = 0.0;
     int32_t probe_iters = 0;
-    bool have_exact = false;   // dense factor of the current matrix is in `dense`
+    bool have_exact = false;   // the factor of the current matrix is in `dense`
     double exact_lhat = 0.0;   // its 2 sum log L_ii
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     // launch accounting and optional SpMM timing
@@ -259,8 +262,8 @@ gp2s_status minres_solve(gp2s_ctx *c, const double *b, double *x, double tol, in
 // columns to relative residual tol (xz: solutions, rz: final recursively updated residuals).
 gp2s_status krylov_columns_buffers(gp2s_ctx *c, int m, void **rz, void **xz);
 gp2s_status krylov_columns_solve(gp2s_ctx *c, int m, double tol, int *iters);
-gp2s_status exact_logdet_solve(gp2s_ctx *c, const double *y_sorted_dev, double *logdet_hat,
-                               bool want_inverse);
+// log|Ah| by tiled Cholesky and, with y_sorted_dev, a = A^{-1} y in vec64 slot 3 (cholesky.cu).
+gp2s_status exact_logdet_solve(gp2s_ctx *c, const double *y_sorted_dev, double *logdet_hat);
 // Reductions used by several stages
 gp2s_status sum_log_diag(gp2s_ctx *c, double *out_host);
 gp2s_status dot_f64(gp2s_ctx *c, const double *a, const double *b, int64_t n, double *out_host);

@@ -4,14 +4,13 @@
 //     relation), and log|Ah| ~= (n/m) sum_s sum_j tau_sj^2 log theta_sj with T_s's eigenvalues theta_j
 //     and eigenvector first components tau_j; the inner sum e_1^T log(T_s) e_1 is evaluated without
 //     them, by the trapezoidal rule on an integral of the logarithm, in FP64.
-//   * EXACT: dense FP64 Cholesky of Ah (right-looking, 32-wide panels: diagonal-block factor,
-//     panel triangular solve, symmetric rank-32 update of the trailing lower triangle), then
-//     log|Ah| = 2 sum log L_ii and the y solve by forward/backward substitution.
+//   * EXACT: FP64 Cholesky of Ah by tiles (cholesky.cu), log|Ah| = 2 sum log L_ii and the y solve.
 //   log|A| = sum log D_ii + log|Ah| in both cases.
 #include <cmath>
 #include <cstring>
 #include <mutex>
 
+#include "gp2s_cholesky.cuh"
 #include "gp2s_internal.cuh"
 #include "gp2s_kernel_math.cuh"
 
@@ -154,181 +153,6 @@ __global__ void k_dot64(const double *__restrict__ a, const double *__restrict__
     }
 }
 
-// ---------------------------------------------------------------------------------------------
-// Dense FP64 Cholesky (lower, column-major-free: row-major n x n, only the lower triangle used)
-// ---------------------------------------------------------------------------------------------
-constexpr int NB = 32;
-
-__global__ void k_densify(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col,
-                          const double *__restrict__ val, int64_t n, double *__restrict__ Ad)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t i = w0; i < n; i += nw)
-        for (int p = rowptr[i] + lane; p < rowptr[i + 1]; p += 32) Ad[i * n + col[p]] = val[p];
-}
-
-// Factor the NB x NB diagonal block at (kb, kb) in shared memory.
-__global__ void k_potrf_diag(double *__restrict__ Ad, int64_t n, int kb, int *__restrict__ bad)
-{
-    __shared__ double S[NB][NB + 1];
-    const int nbk = (int)(n - kb < NB ? n - kb : NB);
-    for (int t = threadIdx.x; t < NB * NB; t += blockDim.x) {
-        int i = t / NB, j = t % NB;
-        S[i][j] = (i < nbk && j < nbk) ? Ad[(int64_t)(kb + i) * n + kb + j] : 0.0;
-    }
-    __syncthreads();
-    for (int j = 0; j < nbk; ++j) {
-        if (threadIdx.x == 0) {
-            double d = S[j][j];
-            if (!(d > 0.0)) { atomicOr(bad, 1); d = 1.0; }
-            S[j][j] = sqrt(d);
-        }
-        __syncthreads();
-        for (int i = j + 1 + threadIdx.x; i < nbk; i += blockDim.x) S[i][j] /= S[j][j];
-        __syncthreads();
-        for (int t = threadIdx.x; t < nbk * nbk; t += blockDim.x) {
-            int i = t / nbk, l = t % nbk;
-            if (i > j && l > j && l <= i) S[i][l] -= S[i][j] * S[l][j];
-        }
-        __syncthreads();
-    }
-    for (int t = threadIdx.x; t < nbk * nbk; t += blockDim.x) {
-        int i = t / nbk, j = t % nbk;
-        if (j <= i) Ad[(int64_t)(kb + i) * n + kb + j] = S[i][j];
-    }
-}
-
-// Panel: rows r >= kb + NB, columns kb..kb+NB: L21 = A21 L11^{-T}.  One thread per row.
-__global__ void k_trsm_panel(double *__restrict__ Ad, int64_t n, int kb)
-{
-    __shared__ double Lk[NB][NB + 1];
-    const int nbk = (int)(n - kb < NB ? n - kb : NB);
-    for (int t = threadIdx.x; t < NB * NB; t += blockDim.x) {
-        int i = t / NB, j = t % NB;
-        Lk[i][j] = (i < nbk && j <= i) ? Ad[(int64_t)(kb + i) * n + kb + j] : 0.0;
-    }
-    __syncthreads();
-    int64_t r = kb + nbk + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n) return;
-    double x[NB];
-    double *row = Ad + r * n + kb;
-    for (int j = 0; j < nbk; ++j) {
-        double v = row[j];
-        for (int l = 0; l < j; ++l) v -= x[l] * Lk[j][l];
-        x[j] = v / Lk[j][j];
-    }
-    for (int j = 0; j < nbk; ++j) row[j] = x[j];
-}
-
-// Trailing update of the lower triangle: A[i][j] -= sum_l L[i][kb+l] L[j][kb+l] for
-// i >= j >= kb + NB.  64 x 64 output tiles, 256 threads, 4 x 4 outputs per thread.
-__global__ void __launch_bounds__(256) k_syrk(double *__restrict__ Ad, int64_t n, int kb)
-{
-    const int64_t t0 = kb + NB;
-    const int64_t ti = t0 + (int64_t)blockIdx.y * 64, tj = t0 + (int64_t)blockIdx.x * 64;
-    if (tj > ti + 63) return;   // strictly upper tile
-    __shared__ double Li[64][NB + 1], Lj[64][NB + 1];
-    const int nbk = (int)(n - kb < NB ? n - kb : NB);
-    for (int t = threadIdx.x; t < 64 * NB; t += blockDim.x) {
-        int r = t / NB, l = t % NB;
-        Li[r][l] = (ti + r < n && l < nbk) ? Ad[(ti + r) * n + kb + l] : 0.0;
-        Lj[r][l] = (tj + r < n && l < nbk) ? Ad[(tj + r) * n + kb + l] : 0.0;
-    }
-    __syncthreads();
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    double acc[4][4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
-    for (int l = 0; l < nbk; ++l) {
-        double vi[4], vj[4];
-#pragma unroll
-        for (int a = 0; a < 4; ++a) { vi[a] = Li[ty + 16 * a][l]; vj[a] = Lj[tx + 16 * a][l]; }
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) acc[a][b] = fma(vi[a], vj[b], acc[a][b]);
-    }
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            int64_t i = ti + ty + 16 * a, j = tj + tx + 16 * b;
-            if (i < n && j <= i) Ad[i * n + j] -= acc[a][b];
-        }
-}
-
-__global__ void k_logdiag(const double *__restrict__ Ad, int64_t n, double *__restrict__ part)
-{
-    __shared__ double sh[32];
-    double s = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        s += log(Ad[i * n + i]);
-    s = warp_sum_d(s);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sh[w];
-        part[blockIdx.x] = t;
-    }
-}
-
-// Forward substitution L z = b, block kb: solve the NB x NB diagonal block (one CTA).
-__global__ void k_trsv_diag(const double *__restrict__ Ad, int64_t n, int kb, double *__restrict__ x, int trans)
-{
-    __shared__ double xs[NB];
-    const int nbk = (int)(n - kb < NB ? n - kb : NB);
-    if (threadIdx.x == 0) {
-        if (!trans) {
-            for (int j = 0; j < nbk; ++j) {
-                double v = x[kb + j];
-                for (int l = 0; l < j; ++l) v -= Ad[(int64_t)(kb + j) * n + kb + l] * xs[l];
-                xs[j] = v / Ad[(int64_t)(kb + j) * n + kb + j];
-            }
-        } else {
-            for (int j = nbk - 1; j >= 0; --j) {
-                double v = x[kb + j];
-                for (int l = j + 1; l < nbk; ++l) v -= Ad[(int64_t)(kb + l) * n + kb + j] * xs[l];
-                xs[j] = v / Ad[(int64_t)(kb + j) * n + kb + j];
-            }
-        }
-        for (int j = 0; j < nbk; ++j) x[kb + j] = xs[j];
-    }
-}
-
-// Forward: x[i] -= sum_l L[i][kb+l] x[kb+l] for i >= kb + NB (one warp per row).
-// Backward (trans): x[j] -= sum_l L[kb+l][j] x[kb+l] for j < kb (one thread per column j).
-__global__ void k_trsv_update(const double *__restrict__ Ad, int64_t n, int kb, double *__restrict__ x, int trans)
-{
-    const int nbk = (int)(n - kb < NB ? n - kb : NB);
-    if (!trans) {
-        const int lane = threadIdx.x & 31;
-        const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-        const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-        for (int64_t i = kb + nbk + w0; i < n; i += nw) {
-            double v = lane < nbk ? Ad[i * n + kb + lane] * x[kb + lane] : 0.0;
-            v = warp_sum_d(v);
-            if (lane == 0) x[i] -= v;
-        }
-    } else {
-        for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < kb; j += (int64_t)gridDim.x * blockDim.x) {
-            double v = 0.0;
-            for (int l = 0; l < nbk; ++l) v = fma(Ad[(int64_t)(kb + l) * n + j], x[kb + l], v);
-            x[j] -= v;
-        }
-    }
-}
-
-__global__ void k_gp2s_mul(int64_t n, const double *a, const double *b, double *out)
-{
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = a[i] * b[i];
-}
-
 gp2s_status reduce_parts(gp2s_ctx *c, const double *part, int cnt, double *out_host)
 {
     std::vector<double> h(cnt);
@@ -442,84 +266,6 @@ gp2s_status slq_logdet(gp2s_ctx *c, int m, int ksteps, double *logdet_hat, doubl
     return GP2S_OK;
 }
 
-gp2s_status exact_logdet_solve(gp2s_ctx *c, const double *y_sorted_dev, double *logdet_hat, bool want_inverse)
-{
-    (void)want_inverse;
-    const Assembled &A = c->A;
-    const int64_t n = A.n;
-    const size_t bytes = sizeof(double) * (size_t)n * (size_t)n;
-    GP2S_TRY(ensure(c, c->dense, bytes + 64));
-    double *Ad = c->dense.as<double>();
-    GP2S_CUDA(c, cudaMemsetAsync(Ad, 0, bytes, c->stream));
-    {
-        unsigned gb = (unsigned)std::min<int64_t>(ceil_div(n * 32, 256), 152 * 16);
-        k_densify<<<gb, 256, 0, c->stream>>>(c->rowptr.as<int32_t>(), c->col.as<int32_t>(), c->val64.as<double>(), n, Ad);
-        GP2S_LAUNCH(c);
-    }
-    GP2S_TRY(ensure(c, c->counters, 256));
-    int *bad = reinterpret_cast<int *>(c->counters.as<char>() + 192);
-    GP2S_CUDA(c, cudaMemsetAsync(bad, 0, sizeof(int), c->stream));
-    for (int64_t kb = 0; kb < n; kb += NB) {
-        k_potrf_diag<<<1, 256, 0, c->stream>>>(Ad, n, (int)kb, bad);
-        GP2S_LAUNCH(c);
-        int64_t rest = n - kb - NB;
-        if (rest > 0) {
-            k_trsm_panel<<<(unsigned)ceil_div(rest, 64), 64, 0, c->stream>>>(Ad, n, (int)kb);
-            GP2S_LAUNCH(c);
-            unsigned tiles = (unsigned)ceil_div(rest, 64);
-            k_syrk<<<dim3(tiles, tiles), 256, 0, c->stream>>>(Ad, n, (int)kb);
-            GP2S_LAUNCH(c);
-        }
-    }
-    int hbad = 0;
-    GP2S_CUDA(c, cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    GP2S_CUDA(c, cudaStreamSynchronize(c->stream));
-    if (hbad) return set_err(c, GP2S_ENOTPD, "dense Cholesky: non-positive pivot");
-    const int nb = 152 * 2;
-    GP2S_TRY(ensure(c, c->gpart, sizeof(double) * (2 * nb + 8)));
-    k_logdiag<<<nb, 256, 0, c->stream>>>(Ad, n, c->gpart.as<double>());
-    GP2S_LAUNCH(c);
-    double half = 0.0;
-    GP2S_TRY(reduce_parts(c, c->gpart.as<double>(), nb, &half));
-    *logdet_hat = 2.0 * half;
-    c->have_exact = true;
-    c->exact_lhat = *logdet_hat;
-
-    if (y_sorted_dev) {
-        // a = s * (Ah^{-1} (s * y)) by forward / backward substitution in vec64 slot 3
-        GP2S_TRY(ensure(c, c->vec64, sizeof(double) * (size_t)n * 4 + 256));
-        double *b64 = c->vec64.as<double>();
-        double *xh = b64 + n, *a64 = b64 + 3 * n;
-        GP2S_TRY(ensure(c, c->gpart, sizeof(double) * (2 * nb + 8)));
-        const unsigned gbn = (unsigned)std::min<int64_t>(ceil_div(n, 256), 152 * 8);
-        // b64 = s * y ; xh = b64
-        k_gp2s_mul<<<gbn, 256, 0, c->stream>>>(n, c->s64.as<double>(), y_sorted_dev, b64);
-        GP2S_LAUNCH(c);
-        GP2S_CUDA(c, cudaMemcpyAsync(xh, b64, sizeof(double) * n, cudaMemcpyDeviceToDevice, c->stream));
-        const unsigned gbu = (unsigned)std::min<int64_t>(ceil_div(n * 32, 256), 152 * 8);
-        for (int64_t kb = 0; kb < n; kb += NB) {
-            k_trsv_diag<<<1, 32, 0, c->stream>>>(Ad, n, (int)kb, xh, 0);
-            GP2S_LAUNCH(c);
-            if (kb + NB < n) {
-                k_trsv_update<<<gbu, 256, 0, c->stream>>>(Ad, n, (int)kb, xh, 0);
-                GP2S_LAUNCH(c);
-            }
-        }
-        for (int64_t kb = ((n - 1) / NB) * NB; kb >= 0; kb -= NB) {
-            k_trsv_diag<<<1, 32, 0, c->stream>>>(Ad, n, (int)kb, xh, 1);
-            GP2S_LAUNCH(c);
-            if (kb > 0) {
-                k_trsv_update<<<gbn, 256, 0, c->stream>>>(Ad, n, (int)kb, xh, 1);
-                GP2S_LAUNCH(c);
-            }
-        }
-        k_gp2s_mul<<<gbn, 256, 0, c->stream>>>(n, c->s64.as<double>(), xh, a64);
-        GP2S_LAUNCH(c);
-        c->have_solution = true;
-    }
-    return GP2S_OK;
-}
-
 }  // namespace gp2s
 
 // =============================================================================================
@@ -528,21 +274,23 @@ gp2s_status exact_logdet_solve(gp2s_ctx *c, const double *y_sorted_dev, double *
 // For callers that may not allocate device memory (work issued during CUDA stream capture, or a
 // device whose memory is owned by another allocator), every intermediate of this path lives in one
 // fixed array compiled into the library.  The dense matrix is built pair by pair with the same
-// exact FP64 support test and FP64 kernel value as the CSR path, then factored by the same blocked
-// Cholesky kernels as the EXACT log-determinant above.
+// exact FP64 support test and FP64 kernel value as the CSR path, then factored by the same tiled
+// Cholesky kernel as the EXACT log-determinant (cholesky.cu), with every tile present.
 // =============================================================================================
 namespace gp2s {
 
 namespace {
 
 constexpr int kNoAllocMaxN = GP2S_NOALLOC_MAX_N;
-constexpr size_t kNoAllocA = (size_t)kNoAllocMaxN * kNoAllocMaxN;              // dense A / its factor
-constexpr size_t kNoAllocX = kNoAllocA;                                          // y, then a = A^{-1} y
-constexpr size_t kNoAllocB = kNoAllocX + kNoAllocMaxN;                           // bump table n x L
-constexpr size_t kNoAllocFlag = kNoAllocB + (size_t)kNoAllocMaxN * kMaxBumps;    // pivot flag (int)
-constexpr size_t kNoAllocDoubles = kNoAllocFlag + 32;
+constexpr int kNoAllocNT = kNoAllocMaxN / kCT;                                   // tile rows
+constexpr int kNoAllocTiles = kNoAllocNT * (kNoAllocNT + 1) / 2;
+constexpr size_t kNoAllocVec = (size_t)kNoAllocTiles * kCTElems;                 // 1 / diag(L), y', x', a (4 n)
+constexpr size_t kNoAllocB = kNoAllocVec + 4 * kNoAllocMaxN;                     // bump table n x L
+constexpr size_t kNoAllocFlag = kNoAllocB + (size_t)kNoAllocMaxN * kMaxBumps;    // tile flags and the pivot flag (int)
+constexpr size_t kNoAllocDoubles = kNoAllocFlag + 128;
+static_assert(kNoAllocMaxN % kCT == 0 && kNoAllocTiles + 2 * kNoAllocNT + 3 <= 256, "the flags fit their place");
 
-// The scratch array: every call on a device shares it (about 2.1 MB per device).
+// The scratch array: every call on a device shares it (about 1.3 MB per device).
 static __device__ __align__(256) double g_noalloc_scratch[kNoAllocDoubles];
 
 std::mutex g_noalloc_mu;
@@ -567,40 +315,52 @@ __global__ void k_noalloc_bumps(const double *__restrict__ X, int n, KernelParam
     }
 }
 
-// Lower triangle of the dense A = K + sigma2 I (every entry written, so no clearing is needed).
+// Slot of tile (i, j), i >= j, of the packed lower triangle of nt x nt tiles (columns one after the other).
+__host__ __device__ inline int noalloc_slot(int nt, int i, int j) { return j * nt - j * (j - 1) / 2 + (i - j); }
+
+// The lower triangle of A = K + sigma2 I in tiles, rows past n as identity rows (every element is
+// written, so no clearing is needed).  One CTA per tile.
 template <int D>
-__global__ void k_noalloc_dense(const double *__restrict__ X, int n, KernelParams kp, const double *__restrict__ B,
-                                double *__restrict__ A)
+__global__ void k_noalloc_tiles(const double *__restrict__ X, int n, int nt, KernelParams kp,
+                                const double *__restrict__ B, double *__restrict__ tiles)
 {
-    const int64_t tot = (int64_t)n * n;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
-        const int i = (int)(e / n), j = (int)(e - (int64_t)i * n);
-        if (j > i) continue;
-        double q = 0.0;
+    int tj = 0, at = blockIdx.x;
+    while (at >= nt - tj) {
+        at -= nt - tj;
+        ++tj;
+    }
+    const int ti = tj + at;
+    for (int e = threadIdx.x; e < kCTElems; e += blockDim.x) {
+        const int i = ti * kCT + e / kCT, j = tj * kCT + e % kCT;
+        double v = i == j ? 1.0 : 0.0;
+        if (i < n && j <= i) {
+            double q = 0.0;
 #pragma unroll
-        for (int k = 0; k < D; ++k) {
-            double dk = __dsub_rn(X[(int64_t)i * D + k], X[(int64_t)j * D + k]);
-            q = __dadd_rn(q, __dmul_rn(dk, dk));
+            for (int k = 0; k < D; ++k) {
+                double dk = __dsub_rn(X[(int64_t)i * D + k], X[(int64_t)j * D + k]);
+                q = __dadd_rn(q, __dmul_rn(dk, dk));
+            }
+            v = 0.0;
+            if (i == j || q < kp.r * kp.r) {
+                double S = 0.0;
+                for (int l = 0; l < kp.L; ++l) S = fma(B[(int64_t)i * kp.L + l], B[(int64_t)j * kp.L + l], S);
+                v = wendland<double>(kp.kind, D, sqrt(q) * kp.inv_r) * (S + kp.w0);
+                if (i == j) v += kp.sigma2;
+            }
         }
-        double v = 0.0;
-        if (i == j || q < kp.r * kp.r) {
-            double S = 0.0;
-            for (int l = 0; l < kp.L; ++l) S = fma(B[(int64_t)i * kp.L + l], B[(int64_t)j * kp.L + l], S);
-            v = wendland<double>(kp.kind, D, sqrt(q) * kp.inv_r) * (S + kp.w0);
-            if (i == j) v += kp.sigma2;
-        }
-        A[e] = v;
+        tiles[(size_t)blockIdx.x * kCTElems + e] = v;
     }
 }
 
 // {LML, y^T a, log|A|} from the factor's diagonal and the solution; NaN when a pivot failed.
-__global__ void k_noalloc_finish(const double *__restrict__ A, int n, const double *__restrict__ y,
+__global__ void k_noalloc_finish(const double *__restrict__ tiles, int n, int nt, const double *__restrict__ y,
                                  const double *__restrict__ a, const int *__restrict__ bad, double *__restrict__ out)
 {
     __shared__ double sh[2][32];
     double ld = 0.0, qd = 0.0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        ld += log(A[(int64_t)i * n + i]);
+        const int j = i / kCT, r = i % kCT;
+        ld += log(tiles[(size_t)noalloc_slot(nt, j, j) * kCTElems + r * kCT + r]);
         qd = fma(y[i], a[i], qd);
     }
     ld = warp_sum_d(ld);
@@ -640,12 +400,10 @@ gp2s_status noalloc_scratch(double **ptr)
 }
 
 template <int D>
-void launch_noalloc_build(const double *X, int n, const KernelParams &kp, double *B, double *A, cudaStream_t s)
+void launch_noalloc_build(const double *X, int n, int nt, const KernelParams &kp, double *B, double *tiles, cudaStream_t s)
 {
     k_noalloc_bumps<D><<<(n + 127) / 128, 128, 0, s>>>(X, n, kp, B);
-    const int64_t tot = (int64_t)n * n;
-    unsigned gb = (unsigned)((tot + 255) / 256 < 4096 ? (tot + 255) / 256 : 4096);
-    k_noalloc_dense<D><<<gb, 256, 0, s>>>(X, n, kp, B, A);
+    k_noalloc_tiles<D><<<chol_dense_tiles(nt), 256, 0, s>>>(X, n, nt, kp, B, tiles);
 }
 
 }  // namespace
@@ -689,41 +447,32 @@ extern "C" gp2s_status gp2s_lml_exact_noalloc(int64_t n, const double *X_dev, co
     if (st != GP2S_OK) return st;
     const int nn = (int)n;
     const KernelParams kp = make_kernel_params(hyper);
-    double *A = base;                          // nn x nn, leading dimension nn
-    double *x = base + kNoAllocX;
+    // A's tiles, factored in place; a = A^{-1} y in the last of the four vectors
+    CholArgs ca{};
+    ca.nt = (nn + kCT - 1) / kCT;
+    ca.ntiles = chol_dense_tiles(ca.nt);
+    ca.ntasks = ca.ntiles + 2 * ca.nt;
+    ca.n = nn;
+    ca.solve = 1;
+    ca.tiles = base;
+    ca.dinv = base + kNoAllocVec;
+    ca.yv = ca.dinv + kNoAllocMaxN;
+    ca.xv = ca.yv + kNoAllocMaxN;
+    ca.x = ca.xv + kNoAllocMaxN;
+    ca.b = y_dev;
+    ca.flags = reinterpret_cast<int *>(base + kNoAllocFlag);
+    const size_t flags = chol_flag_ints(ca.ntiles, ca.nt);
+    ca.bad = ca.flags + flags;
     double *B = base + kNoAllocB;
-    int *bad = reinterpret_cast<int *>(base + kNoAllocFlag);
-    if (cudaMemsetAsync(bad, 0, sizeof(int), s) != cudaSuccess) { cudaGetLastError(); return GP2S_ECUDA; }
-    if (cudaMemcpyAsync(x, y_dev, sizeof(double) * nn, cudaMemcpyDeviceToDevice, s) != cudaSuccess) {
-        cudaGetLastError();
-        return GP2S_ECUDA;
-    }
+    if (cudaMemsetAsync(ca.flags, 0, sizeof(int) * (flags + 1), s) != cudaSuccess) { cudaGetLastError(); return GP2S_ECUDA; }
     switch (hyper->d) {
-    case 1: launch_noalloc_build<1>(X_dev, nn, kp, B, A, s); break;
-    case 2: launch_noalloc_build<2>(X_dev, nn, kp, B, A, s); break;
-    case 3: launch_noalloc_build<3>(X_dev, nn, kp, B, A, s); break;
-    default: launch_noalloc_build<4>(X_dev, nn, kp, B, A, s); break;
+    case 1: launch_noalloc_build<1>(X_dev, nn, ca.nt, kp, B, ca.tiles, s); break;
+    case 2: launch_noalloc_build<2>(X_dev, nn, ca.nt, kp, B, ca.tiles, s); break;
+    case 3: launch_noalloc_build<3>(X_dev, nn, ca.nt, kp, B, ca.tiles, s); break;
+    default: launch_noalloc_build<4>(X_dev, nn, ca.nt, kp, B, ca.tiles, s); break;
     }
-    // blocked Cholesky A = L L^T (lower triangle, in place)
-    for (int kb = 0; kb < nn; kb += NB) {
-        k_potrf_diag<<<1, 256, 0, s>>>(A, nn, kb, bad);
-        int rest = nn - kb - NB;
-        if (rest > 0) {
-            k_trsm_panel<<<(rest + 63) / 64, 64, 0, s>>>(A, nn, kb);
-            unsigned tiles = (unsigned)((rest + 63) / 64);
-            k_syrk<<<dim3(tiles, tiles), 256, 0, s>>>(A, nn, kb);
-        }
-    }
-    // a = L^{-T} L^{-1} y, in place in x
-    for (int kb = 0; kb < nn; kb += NB) {
-        k_trsv_diag<<<1, 32, 0, s>>>(A, nn, kb, x, 0);
-        if (kb + NB < nn) k_trsv_update<<<(unsigned)((nn * 32 + 255) / 256), 256, 0, s>>>(A, nn, kb, x, 0);
-    }
-    for (int kb = ((nn - 1) / NB) * NB; kb >= 0; kb -= NB) {
-        k_trsv_diag<<<1, 32, 0, s>>>(A, nn, kb, x, 1);
-        if (kb > 0) k_trsv_update<<<(unsigned)((kb + 255) / 256), 256, 0, s>>>(A, nn, kb, x, 1);
-    }
-    k_noalloc_finish<<<1, 256, 0, s>>>(A, nn, y_dev, x, bad, out_dev);
+    if (chol_launch(ca, 152, s) != cudaSuccess) return GP2S_ECUDA;
+    k_noalloc_finish<<<1, 256, 0, s>>>(ca.tiles, nn, ca.nt, y_dev, ca.x, ca.bad, out_dev);
     if (cudaGetLastError() != cudaSuccess) return GP2S_ECUDA;
     return GP2S_OK;
 }

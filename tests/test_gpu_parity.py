@@ -295,6 +295,22 @@ def test_logdet_slq_matches_oracle_with_identical_probes(gp, ctx, precond):
     assert abs(info["logdet"] - e["logdet"]) <= 5 * info["logdet_stderr"] + 1e-9 * abs(e["logdet"])
 
 
+@pytest.mark.parametrize("n,d,r", [(1, 1, 0.1), (2, 2, 2.0), (31, 1, 0.05), (32, 2, 2.0), (33, 3, 0.3), (64, 1, 0.02), (65, 2, 0.1),
+                                   (97, 3, 2.0), (513, 1, 0.004), (1000, 1, 0.03), (1025, 2, 0.05), (2111, 3, 0.12)])
+def test_tiled_cholesky_at_tile_edges(gp, ctx, n, d, r):
+    """The exact log-determinant and solve by 32-row tiles: one row, sizes around a tile and several
+    tiles, a diagonal-like and a banded matrix, a full one (r = 2), tile fill in 2-D and 3-D.  FP64 on both
+    sides: n^2 products of rounding 1.1e-16, a condition number of at most a few 1e3 on the log scale."""
+    import oracle
+    w = W.random_small(700 + n, n, d, L=3, sigma2=1e-2, r=r)
+    opts = gp.default_opts(precision=gp.PREC_FP64, logdet=gp.LOGDET_EXACT)
+    lml, info = ctx.lml(w["X"], w["y"], gp.Hyper(**w["hyper"]), opts)
+    e = oracle.lml_exact(w["X"], w["y"], oracle.Hyper(**w["hyper"]))
+    assert info["logdet"] == pytest.approx(e["logdet"], rel=1e-10, abs=1e-10 * n)
+    assert info["quad"] == pytest.approx(e["quad"], rel=1e-10)
+    assert lml == pytest.approx(e["lml"], rel=1e-10, abs=1e-9)
+
+
 @pytest.mark.parametrize("steps,rel", [(1, 1e-9), (2, 1e-9), (33, 1e-9), (257, 1e-6), (300, 1e-6)])
 def test_slq_quadrature_matches_the_oracle_eigensolve(gp, ctx, steps, rel):
     """The quadrature of log T without its eigen-decomposition against the oracle's Gauss quadrature, in

@@ -78,6 +78,19 @@ def test_noalloc_matches_the_oracle(gp, d, kind, w0):
     assert out[0] == pytest.approx(e["lml"], rel=1e-8)
 
 
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 480, 511, 512])
+def test_noalloc_at_tile_edges(gp, n):
+    """Sizes around the 32-row tiles of the factorisation, against the oracle (FP64 on both sides)."""
+    import oracle
+    w = W.random_small(420 + n, n, 2, L=2, sigma2=1e-2, r=0.3)
+    X = torch.tensor(w["X"], dtype=torch.float64, device="cuda")
+    y = torch.tensor(w["y"], dtype=torch.float64, device="cuda")
+    st, out = _noalloc(gp, X, y, gp.Hyper(**w["hyper"]))
+    assert st == gp.OK
+    e = oracle.lml_exact(w["X"], w["y"], oracle.Hyper(**w["hyper"]))
+    assert out == pytest.approx([e["lml"], e["quad"], e["logdet"]], rel=1e-10, abs=1e-10 * n)
+
+
 def test_noalloc_rejects_sizes_beyond_the_limit(gp):
     w = W.random_small(403, 513, 2)
     h = gp.Hyper(**w["hyper"])
