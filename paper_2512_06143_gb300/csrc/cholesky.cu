@@ -375,6 +375,7 @@ k_chol(const CholArgs a)
                 double v;
                 if (fw) v = o + lane < a.n ? (a.bs ? a.bs[o + lane] : 1.0) * a.b[o + lane] : 0.0;
                 else v = __ldcg(a.yv + j * kCT + lane);
+                if (fw && a.bh && o + lane < a.n) a.bh[o + lane] = v;
                 v -= vec[lane];
                 if (fw) {
 #pragma unroll 8
@@ -392,7 +393,10 @@ k_chol(const CholArgs a)
                         else if (lane < c) v = fma(-x, Bs_[c][lane], v);
                     }
                     a.xv[j * kCT + lane] = v;
-                    if (o + lane < a.n) a.x[o + lane] = (a.bs ? a.bs[o + lane] : 1.0) * v;
+                    if (o + lane < a.n) {
+                        a.x[o + lane] = (a.bs ? a.bs[o + lane] : 1.0) * v;
+                        if (a.xh) a.xh[o + lane] = v;
+                    }
                 }
             }
             finish((fw ? done_y : done_x) + j);
@@ -657,10 +661,14 @@ gp2s_status exact_logdet_solve(gp2s_ctx *c, const double *y_sorted_dev, double *
     const unsigned gb = (unsigned)std::min<int64_t>(ceil_div((int64_t)nv * 32, 256), 152 * 16);
     k_chol_fill<<<gb, 256, 0, c->stream>>>(c->rowptr.as<int32_t>(), c->col.as<int32_t>(), c->val64.as<double>(), n, a, pos);
     GP2S_LAUNCH(c);
-    // a = s * (Ah^{-1} (s * y)), vec64 slot 3
+    // a = s * (Ah^{-1} (s * y)), vec64 slot 3; slots 0 and 1 hold s * y and Ah^{-1} (s * y) for the residual
     a.b = y_sorted_dev;
     a.bs = c->s64.as<double>();
-    a.x = a.solve ? c->vec64.as<double>() + 3 * n : nullptr;
+    if (a.solve) {
+        a.bh = c->vec64.as<double>();
+        a.xh = a.bh + n;
+        a.x = a.bh + 3 * n;
+    }
     ++c->launches;
     GP2S_CUDA(c, chol_launch(a, c->num_sms, c->stream));
     const int nb = 64;

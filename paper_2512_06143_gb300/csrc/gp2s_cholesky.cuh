@@ -27,6 +27,7 @@ struct CholArgs {
     const double *bs;
     double *yv, *xv;             // nt x kCT each: forward and backward solutions (elimination order)
     double *x;                   // n (unpermuted): the solution, scaled by bs
+    double *bh, *xh;             // n (unpermuted), optional: bs * b and the solution before its scaling
     int *flags;                  // ntiles + 2 nt finished marks, then the ticket counter and the abort word
     int *bad;                    // bit 0: a pivot was not positive, bit 1: a bounded wait gave up
 };

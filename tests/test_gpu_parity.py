@@ -309,6 +309,7 @@ def test_tiled_cholesky_at_tile_edges(gp, ctx, n, d, r):
     assert info["logdet"] == pytest.approx(e["logdet"], rel=1e-10, abs=1e-10 * n)
     assert info["quad"] == pytest.approx(e["quad"], rel=1e-10)
     assert lml == pytest.approx(e["lml"], rel=1e-10, abs=1e-9)
+    assert info["relres"] <= 1e-12      # the residual is formed from this call's right-hand side and solution
 
 
 @pytest.mark.parametrize("steps,rel", [(1, 1e-9), (2, 1e-9), (33, 1e-9), (257, 1e-6), (300, 1e-6)])
