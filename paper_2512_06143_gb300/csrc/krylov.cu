@@ -287,7 +287,7 @@ __device__ __forceinline__ double block_sum(const double *__restrict__ p, int cn
 {
     __shared__ double sh[32];
     double s = 0.0;
-    for (int b = threadIdx.x; b < cnt; b += blockDim.x) s += p[b];
+    for (int b = threadIdx.x; b < cnt; b += blockDim.x) s += __ldcg(p + b);
     s = warp_sum(s);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
     __syncthreads();
@@ -332,35 +332,78 @@ __global__ void k_scal_init(const double *__restrict__ part, const double *__res
 // residual has already fallen to the rounding level of the vector precision (|r|^2 <= lucky
 // |b|^2): then the Krylov space is exhausted and the column simply stops, with the steps it has
 // recorded (a small problem, or an operator with few distinct eigenvalues).
+__device__ __forceinline__ void scal_alpha(int c, double s, double *__restrict__ sc, int *__restrict__ active,
+                                           int *__restrict__ flags, double *__restrict__ rec, int ksteps, double lucky)
+{
+    double *q = sc + c * kScal;
+    q[S_PQ] = s;
+    if (!active[c]) {
+        q[S_ALPHA] = 0.0;
+        return;
+    }
+    if (!(s > 0.0)) {
+        active[c] = 0;
+        q[S_ALPHA] = 0.0;
+        q[S_STOP] = 2.0;
+        if (!(q[S_RR] <= lucky * q[S_B2])) atomicOr(&flags[0], 1);   // breakdown
+        return;
+    }
+    double a = q[S_RHO] / s;
+    q[S_ALPHA] = a;
+    int st = (int)q[S_STEPS];
+    if (c > 0 && rec && st < ksteps) rec[((int64_t)(c - 1) * ksteps + st) * 2 + 0] = a;
+}
+
 __global__ void k_scal_alpha(const double *__restrict__ part, int pstride, int nparts, double *__restrict__ sc,
                              int *__restrict__ active, int *__restrict__ flags, double *__restrict__ rec,
                              int ksteps, double lucky)
 {
     const int c = blockIdx.x;
     double s = block_sum(part + (int64_t)c * pstride, nparts);
-    if (threadIdx.x == 0) {
-        double *q = sc + c * kScal;
-        q[S_PQ] = s;
-        if (!active[c]) {
-            q[S_ALPHA] = 0.0;
-            return;
-        }
-        if (!(s > 0.0)) {
-            active[c] = 0;
-            q[S_ALPHA] = 0.0;
-            q[S_STOP] = 2.0;
-            if (!(q[S_RR] <= lucky * q[S_B2])) atomicOr(&flags[0], 1);   // breakdown
-            return;
-        }
-        double a = q[S_RHO] / s;
-        q[S_ALPHA] = a;
-        int st = (int)q[S_STEPS];
-        if (c > 0 && rec && st < ksteps) rec[((int64_t)(c - 1) * ksteps + st) * 2 + 0] = a;
-    }
+    if (threadIdx.x == 0) scal_alpha(c, s, sc, active, flags, rec, ksteps, lucky);
 }
 
 // beta_c = rr_c / rho_c, rho_c = rr_c, convergence test |r|^2 <= tol^2 |b|^2 once at least
 // kmin steps are recorded (the probe columns keep iterating to give SLQ its k Lanczos steps).
+__device__ __forceinline__ void scal_beta(int c, double s, double s2, double *__restrict__ sc, int *__restrict__ active,
+                                          int *__restrict__ count, double *__restrict__ rec, int ksteps, int kmin_probe,
+                                          double lucky)
+{
+    double *q = sc + c * kScal;
+    if (!active[c]) {
+        q[S_BETA] = 0.0;
+        return;
+    }
+    q[S_RR] = s2;
+    double b = s / q[S_RHO];
+    int st = (int)q[S_STEPS];
+    if (c > 0 && rec && st < ksteps) rec[((int64_t)(c - 1) * ksteps + st) * 2 + 1] = b;
+    q[S_BETA] = b;
+    q[S_RHO_PREV] = q[S_RHO];
+    q[S_RHO] = s;
+    q[S_STEPS] = (double)(st + 1);
+    bool conv = s2 <= q[S_TOL];
+    int kmin = c == 0 ? 0 : kmin_probe;
+    // a residual at the rounding level ends the column even before kmin steps: the steps after
+    // it would only record rounding noise as Lanczos coefficients
+    const bool exhausted = s2 <= lucky * q[S_B2];
+    if ((conv && st + 1 >= kmin) || exhausted || !(s == s)) {
+        active[c] = 0;
+        q[S_STOP] = 1.0;
+        // p is not updated for inactive columns (beta unused)
+    } else {
+        atomicAdd(count, 1);
+        if (c > 0) atomicAdd(count + 1, 1);
+    }
+}
+
+// p of the y column: the buffer that flags[7] names (YFuse; always the first one without it).
+template <class T>
+__device__ __forceinline__ const T *y_direction(const T *p0, const T *p1, const int *flags)
+{
+    return flags[7] ? p1 : p0;
+}
+
 __global__ void k_scal_beta(const double *__restrict__ part, const double *__restrict__ part_rr, int pstride,
                             int nparts_y, int nparts_z, double *__restrict__ sc, int *__restrict__ active,
                             int *__restrict__ count, double *__restrict__ rec, int ksteps, int kmin_probe, int pc_y,
@@ -372,34 +415,40 @@ __global__ void k_scal_beta(const double *__restrict__ part, const double *__res
     double s = block_sum(part + (int64_t)c * pstride, np);
     __syncthreads();
     double s2 = pc ? block_sum(part_rr + (int64_t)c * pstride, np) : s;
+    if (threadIdx.x == 0) scal_beta(c, s, s2, sc, active, count, rec, ksteps, kmin_probe, lucky);
+}
+
+// The y column's scalars at the end of the kernel that makes their partial sums (y-only iterations): the CTA
+// that finishes last sums them, in k_scal_alpha's and k_scal_beta's order, and takes the step.  On a small
+// matrix the two scalar launches and the counters' memset were 10 us of a 26 us iteration.
+//
+// With DIR the direction kernel goes as well: beta leaves its update pending (flags[6]), and the next SpMV
+// gathers z + beta p (k_direction's FMA) in place of p, the owner of a row writing the new p into the
+// other of two buffers (flags[7] says which one holds p now).  Two gathers per entry instead of one and a
+// launch: taken up to kYDirRows rows, where both vectors (512 KB) stay close to the SMs; at 100,000 rows and
+// more the iteration is bound by the matrix and the launch no longer shows.
+// An iteration of six launches took 21.4 us at n = 2,500 (1-D), 24.3 us at 12,452 rows of 168 entries; with
+// the scalars fused 18.6 and 22.9 us, with the direction too 17.0 and 21.4 us.
+struct YFuse {
+    double *sc = nullptr;      // nullptr: the scalar kernels follow as launches of their own
+    int *active, *flags;       // flags[4], [5]: CTAs finished (alpha, beta); zero between launches
+    double lucky;
+    int dir = 0;               // the direction update is left to the next SpMV
+};
+constexpr int64_t kYDirRows = 1 << 16;
+
+// Called by every thread of the CTA once its partial sums are written (by thread 0): true in the CTA that
+// finishes last.
+__device__ __forceinline__ bool last_cta(int *counter, int ctas)
+{
+    __shared__ int last;
     if (threadIdx.x == 0) {
-        double *q = sc + c * kScal;
-        if (!active[c]) {
-            q[S_BETA] = 0.0;
-            return;
-        }
-        q[S_RR] = s2;
-        double b = s / q[S_RHO];
-        int st = (int)q[S_STEPS];
-        if (c > 0 && rec && st < ksteps) rec[((int64_t)(c - 1) * ksteps + st) * 2 + 1] = b;
-        q[S_BETA] = b;
-        q[S_RHO_PREV] = q[S_RHO];
-        q[S_RHO] = s;
-        q[S_STEPS] = (double)(st + 1);
-        bool conv = s2 <= q[S_TOL];
-        int kmin = c == 0 ? 0 : kmin_probe;
-        // a residual at the rounding level ends the column even before kmin steps: the steps after
-        // it would only record rounding noise as Lanczos coefficients
-        const bool exhausted = s2 <= lucky * q[S_B2];
-        if ((conv && st + 1 >= kmin) || exhausted || !(s == s)) {
-            active[c] = 0;
-            q[S_STOP] = 1.0;
-            // p is not updated for inactive columns (beta unused)
-        } else {
-            atomicAdd(count, 1);
-            if (c > 0) atomicAdd(count + 1, 1);
-        }
+        __threadfence();
+        last = atomicAdd(counter, 1) == ctas - 1;
     }
+    __syncthreads();
+    if (last) __threadfence();
+    return last != 0;
 }
 
 // Restart of the probe columns as PCG: rho = r^T z for the still active columns.
@@ -485,7 +534,7 @@ template <class T>
 __global__ void k_update(int64_t n, int m, T *__restrict__ xz, T *__restrict__ rz, const T *__restrict__ pz,
                          const T *__restrict__ qz, T *__restrict__ xy, T *__restrict__ ry, const T *__restrict__ py,
                          const T *__restrict__ qy, const double *__restrict__ sc, double *__restrict__ part,
-                         int pstride, int nbz)
+                         int pstride, int nbz, YFuse f, const T *__restrict__ py2)
 {
     using Acc = typename AccOf<T>::type;
     __shared__ double shv[kSpmmThreads / 32 + 1][32];
@@ -521,10 +570,11 @@ __global__ void k_update(int64_t n, int m, T *__restrict__ xz, T *__restrict__ r
         const int nby = gridDim.x - nbz;
         const double alpha = sc[0 * kScal + S_ALPHA];
         const T a = (T)alpha;
+        const T *pc = f.dir ? y_direction(py, py2, f.flags) : py;
         for (int64_t i = (int64_t)b * blockDim.x + threadIdx.x; i < n; i += (int64_t)nby * blockDim.x) {
             T r = ry[i];
             if (alpha != 0.0) {
-                xy[i] = xy[i] + a * py[i];
+                xy[i] = xy[i] + a * pc[i];
                 r = r - a * qy[i];
                 ry[i] = r;
             }
@@ -537,6 +587,14 @@ __global__ void k_update(int64_t n, int m, T *__restrict__ xz, T *__restrict__ r
             double s = 0.0;
             for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += shv[w][0];
             part[(int64_t)0 * pstride + b] = s;
+        }
+        if (f.sc && last_cta(&f.flags[5], nby)) {
+            const double s = block_sum(part, nby);
+            if (threadIdx.x == 0) {
+                f.flags[5] = 0;
+                scal_beta(0, s, s, f.sc, f.active, f.flags + 1, nullptr, 0, 0, f.lucky);
+                f.flags[6] = f.dir && f.active[0];
+            }
         }
     }
 }
@@ -695,6 +753,7 @@ __global__ void k_sum_parts(const double *__restrict__ part, int cnt, int groups
 struct CGBuffers {
     void *xz, *rz, *pz, *qz, *xy, *ry, *py, *qy;
     void *zz, *zy;   // preconditioned residuals (block-Jacobi PCG)
+    void *py2;       // the y column's other direction buffer (YFuse)
 };
 
 template <int KH, int NG>
@@ -708,16 +767,30 @@ gp2s_status launch_rb4_et(gp2s_ctx *c, const CGBuffers &B, double *part, int pst
 // loads in flight; per-CTA partial dot p^T q.
 constexpr int kSpmvThreads = 256;
 constexpr int kSpmvBlocks = 152 * 8;
-template <class T, class V>
+template <class T, class V, bool DIR>
 __global__ void __launch_bounds__(kSpmvThreads)
 k_spmv_y(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col, const V *__restrict__ val, int64_t n,
-         const T *__restrict__ py, T *__restrict__ qy, double *__restrict__ part)
+         T *__restrict__ pa, T *__restrict__ pb, const T *__restrict__ z, T *__restrict__ qy, double *__restrict__ part,
+         YFuse f)
 {
     using Acc = typename AccOf<T>::type;
     __shared__ double sh[kSpmvThreads / kWarp];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    // p, and with a pending direction update z + beta p
+    const T *__restrict__ py = pa;
+    T *__restrict__ pn = pb;
+    bool pend = false;
+    T bt = T(0);
+    if (DIR) {
+        if (f.flags[7]) {
+            py = pb;
+            pn = pa;
+        }
+        pend = f.flags[6] != 0;
+        bt = (T)f.sc[S_BETA];
+    }
     Acc d;
     for (int64_t i = w0; i < n; i += nw) {
         const int p1 = rowptr[i + 1];
@@ -735,14 +808,26 @@ k_spmv_y(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col, co
             T g[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) g[u] = py[cj[u]];
+            if (DIR && pend) {
+                T h[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) h[u] = z[cj[u]];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) g[u] = h[u] + bt * g[u];
+            }
 #pragma unroll
             for (int u = 0; u < 4; ++u) s += (T)v[u] * g[u];
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (lane == 0) {
+            T pi = py[i];
+            if (DIR && pend) {
+                pi = z[i] + bt * pi;
+                pn[i] = pi;
+            }
             qy[i] = s;
-            d.fma2(py[i], s);
+            d.fma2(pi, s);
         }
     }
     if (lane == 0) sh[wid] = d.value();
@@ -751,6 +836,18 @@ k_spmv_y(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col, co
         double t = 0.0;
         for (int w = 0; w < kSpmvThreads / kWarp; ++w) t += sh[w];
         part[blockIdx.x] = t;
+    }
+    if (f.sc && last_cta(&f.flags[4], gridDim.x)) {
+        const double s = block_sum(part, gridDim.x);
+        if (threadIdx.x == 0) {
+            f.flags[4] = 0;
+            f.flags[1] = f.flags[2] = 0;     // the active counts that beta makes
+            if (DIR && pend) {
+                f.flags[6] = 0;
+                f.flags[7] ^= 1;
+            }
+            scal_alpha(0, s, f.sc, f.active, f.flags, nullptr, 0, f.lucky);
+        }
     }
 }
 
@@ -781,7 +878,8 @@ __global__ void k_row_split(const int32_t *__restrict__ rowptr, int64_t n, int n
 
 template <class T, class V>
 gp2s_status launch_spmm(gp2s_ctx *c, int m, bool has_y, const V *val, const CGBuffers &B, double *part,
-                        int pstride, int nb, const int32_t *rsplit, const int *active, int *nparts, int *err)
+                        int pstride, int nb, const int32_t *rsplit, const int *active, int *nparts, int *err,
+                        const YFuse &fuse, const T *zy)
 {
     *nparts = nb;
     const Assembled &A = c->A;
@@ -847,7 +945,9 @@ gp2s_status launch_spmm(gp2s_ctx *c, int m, bool has_y, const V *val, const CGBu
     if (has_y && m == 0) {
         const int nbv = (int)std::min<int64_t>(std::min(kSpmvBlocks, pstride),
                                                std::max<int64_t>(1, ceil_div(A.n * kWarp, kSpmvThreads)));
-        k_spmv_y<T, V><<<nbv, kSpmvThreads, 0, c->stream>>>(rp, cl, val, A.n, py, qy, part);
+        T *pa = (T *)B.py, *pb = (T *)B.py2;
+        if (fuse.dir) k_spmv_y<T, V, true><<<nbv, kSpmvThreads, 0, c->stream>>>(rp, cl, val, A.n, pa, pb, zy, qy, part, fuse);
+        else k_spmv_y<T, V, false><<<nbv, kSpmvThreads, 0, c->stream>>>(rp, cl, val, A.n, pa, pb, zy, qy, part, fuse);
         GP2S_LAUNCH(c);
         *nparts = nbv;
         if (ev_b) GP2S_CUDA(c, cudaEventRecord(ev_b, c->stream));
@@ -1875,7 +1975,8 @@ k_pc_step(int64_t n, int m, int64_t nblk, int gz, const float *__restrict__ Minv
           float *__restrict__ rz, float *__restrict__ pz, const float *__restrict__ qz, float *__restrict__ zz,
           float *__restrict__ xy, float *__restrict__ ry, float *__restrict__ py, const float *__restrict__ qy,
           float *__restrict__ zy, const double *__restrict__ rhs_y, const double *__restrict__ sc,
-          double *__restrict__ part_rz, double *__restrict__ part_rr, int pstride, int wy)
+          double *__restrict__ part_rz, double *__restrict__ part_rr, int pstride, int wy, YFuse f,
+          const float *__restrict__ py2)
 {
     constexpr bool SETP = MODE == PC_INIT || MODE == PC_RESTART;   // p = z
     extern __shared__ __align__(16) float pc_sh[];
@@ -2020,6 +2121,7 @@ k_pc_step(int64_t n, int m, int64_t nblk, int gz, const float *__restrict__ Minv
         double arz = 0.0, arr = 0.0;
         const double alpha = MODE == PC_UPDATE ? sc[S_ALPHA] : 0.0;
         const float a = (float)alpha;
+        const float *pc = MODE == PC_UPDATE && f.dir ? y_direction<float>(py, py2, f.flags) : py;
         for (int64_t bg = cb; bg * G < nblk; bg += gy) {
             const int64_t b = bg * G + sub;
             const bool live = b < nblk;
@@ -2039,7 +2141,7 @@ k_pc_step(int64_t n, int m, int64_t nblk, int gz, const float *__restrict__ Minv
                     } else {
                         r = ry[e];
                         if (alpha != 0.0) {
-                            xy[e] = xy[e] + a * py[e];
+                            xy[e] = xy[e] + a * pc[e];
                             r = r - a * qy[e];
                             ry[e] = r;
                         }
@@ -2053,7 +2155,9 @@ k_pc_step(int64_t n, int m, int64_t nblk, int gz, const float *__restrict__ Minv
                 float z = 0.0f;
                 const float *Mb = Minv32 + b * BJ * BJ;
                 const float *Rb = R + sub * BJ;
-#pragma unroll 8
+                // 32 loads of a thread in flight (eight left the y step at 60 % of the HBM rate: 50 us at
+                // 400,000 rows of 128-row blocks, and a solve there 159 us an iteration against 142)
+#pragma unroll 32
                 for (int k = 0; k < BJ; ++k) z = fmaf(__ldcs(Mb + k * BJ + i), Rb[k], z);
                 if (i < nb) {
                     zy[i0 + i] = z;
@@ -2080,6 +2184,16 @@ k_pc_step(int64_t n, int m, int64_t nblk, int gz, const float *__restrict__ Minv
             for (int w = 0; w < kPCThreads / kWarp; ++w) { s1 += red[0][w]; s2 += red[1][w]; }
             part_rz[cb] = s1;
             part_rr[cb] = s2;
+        }
+        if (MODE == PC_UPDATE && f.sc && last_cta(&f.flags[5], gy)) {
+            const double s = block_sum(part_rz, gy);
+            __syncthreads();
+            const double s2 = block_sum(part_rr, gy);
+            if (threadIdx.x == 0) {
+                f.flags[5] = 0;
+                scal_beta(0, s, s2, f.sc, f.active, f.flags + 1, nullptr, 0, 0, f.lucky);
+                f.flags[6] = f.dir && f.active[0];
+            }
         }
     }
 }
@@ -2586,8 +2700,10 @@ gp2s_status cg_run(gp2s_ctx *c, int m, const V *val, const CGBuffers &B, const d
     double *part = c->partials.as<double>();
     double *sc = c->scal.as<double>();
     int *active = reinterpret_cast<int *>(sc + kScal * kMaxCols);
-    int *flags = active + kMaxCols;   // [0] breakdown, [1] active columns, [2] active probe columns
-    GP2S_CUDA(c, cudaMemsetAsync(flags, 0, sizeof(int) * 4, c->stream));
+    // [0] breakdown, [1] active columns, [2] active probe columns, [3] a bounded wait gave up, [4], [5] CTAs
+    // finished, [6] a direction update is pending, [7] which buffer holds the y column's p (YFuse)
+    int *flags = active + kMaxCols;
+    GP2S_CUDA(c, cudaMemsetAsync(flags, 0, sizeof(int) * 8, c->stream));
 
     // Block-Jacobi PCG (FP32 vectors, when the preconditioner is built) or plain CG on Ah.  The y
     // column is preconditioned from the start; the probe columns only when no SLQ records are
@@ -2624,22 +2740,22 @@ gp2s_status cg_run(gp2s_ctx *c, int m, const V *val, const CGBuffers &B, const d
     k_pc_step<MODE, BJ><<<pgz, kPCThreads, pc_smem(MM, BJ), c->stream>>>(                                          \
         n, MM, nblkz, pgz, Minvz, (float *)B.xz, (float *)B.rz, (float *)B.pz, (const float *)B.qz, (float *)B.zz, \
         (float *)B.xy, (float *)B.ry, (float *)B.py, (const float *)B.qy, (float *)B.zy, rhs_y, sc, part, part_rr,  \
-        pstride, WY)
+        pstride, WY, YFuse(), nullptr)
 #define GP2S_PCZ_WY(MODE, MM, WY)                                                                                   \
     do {                                                                                                            \
         if (bjz == 128) GP2S_PCZ_BJ(MODE, 128, MM, WY);                                                             \
         else GP2S_PCZ_BJ(MODE, 64, MM, WY);                                                                         \
     } while (0)
 #define GP2S_PCZ(MODE, MM) GP2S_PCZ_WY(MODE, MM, 0)
-#define GP2S_PCY_BJ(MODE, BJ)                                                                                       \
+#define GP2S_PCY_BJ(MODE, BJ, FUSE)                                                                                       \
     k_pc_step<MODE, BJ><<<pgy, kPCThreads, pc_smem(0, BJ), c->stream>>>(                                           \
         n, 0, nblky, 0, Minvy, (float *)B.xz, (float *)B.rz, (float *)B.pz, (const float *)B.qz, (float *)B.zz,    \
         (float *)B.xy, (float *)B.ry, (float *)B.py, (const float *)B.qy, (float *)B.zy, rhs_y, sc, part, part_rr, \
-        pstride, 0)
-#define GP2S_PCY(MODE)                                                                                              \
+        pstride, 0, FUSE, (const float *)B.py2)
+#define GP2S_PCY(MODE, FUSE)                                                                                        \
     do {                                                                                                            \
-        if (bjy == 128) GP2S_PCY_BJ(MODE, 128);                                                                     \
-        else GP2S_PCY_BJ(MODE, 64);                                                                                 \
+        if (bjy == 128) GP2S_PCY_BJ(MODE, 128, FUSE);                                                               \
+        else GP2S_PCY_BJ(MODE, 64, FUSE);                                                                           \
     } while (0)
     // the probe group's UPDATE step on the warp-specialised bulk-copy kernel (FP32, m = 32 or 64, the
     // instantiated widths; 128-row stages holding one 128-row or two 64-row block-Jacobi blocks):
@@ -2700,7 +2816,7 @@ gp2s_status cg_run(gp2s_ctx *c, int m, const V *val, const CGBuffers &B, const d
                                                       (T *)B.ry, (T *)B.py, part, pstride, nbz);
         GP2S_LAUNCH(c);
     }
-    if (pcy) GP2S_PCY(PC_INIT);
+    if (pcy) GP2S_PCY(PC_INIT, YFuse());
     else k_cg_init<T><<<nby, ut, 0, c->stream>>>(n, m > 0 ? m : 1, rhs_y, (T *)B.xz, (T *)B.rz, (T *)B.pz,
                                                   (T *)B.xy, (T *)B.ry, (T *)B.py, part, pstride, 0);
     GP2S_LAUNCH(c);
@@ -2721,10 +2837,24 @@ gp2s_status cg_run(gp2s_ctx *c, int m, const V *val, const CGBuffers &B, const d
     auto one_iter = [&]() -> gp2s_status {
         const int kc = 1 + mc;
         int np = nb;
-        GP2S_TRY((launch_spmm<T, V>(c, mc, true, val, B, part, pstride, nb, rsplit, active, &np, dev_err)));
-        k_scal_alpha<<<kc, 256, 0, c->stream>>>(part, pstride, np, sc, active, flags, rec, ksteps, lucky);
-        GP2S_LAUNCH(c);
-        GP2S_CUDA(c, cudaMemsetAsync(flags + 1, 0, sizeof(int) * 2, c->stream));
+        const T *zyp = pcy ? (const T *)B.zy : (const T *)B.ry;
+        // y only: alpha and beta are formed at the end of the kernels that make their sums (CTAs of whole
+        // warps: 48 and 96 columns give k_update other sizes)
+        YFuse fuse;
+        const bool fused_scal = mc == 0 && (pcy || ut == 256);
+        if (fused_scal) {
+            fuse.sc = sc;
+            fuse.active = active;
+            fuse.flags = flags;
+            fuse.lucky = lucky;
+            fuse.dir = n <= kYDirRows && !rel;   // a residual replacement continues from p in its own buffer
+        }
+        GP2S_TRY((launch_spmm<T, V>(c, mc, true, val, B, part, pstride, nb, rsplit, active, &np, dev_err, fuse, zyp)));
+        if (!fused_scal) {
+            k_scal_alpha<<<kc, 256, 0, c->stream>>>(part, pstride, np, sc, active, flags, rec, ksteps, lucky);
+            GP2S_LAUNCH(c);
+            GP2S_CUDA(c, cudaMemsetAsync(flags + 1, 0, sizeof(int) * 2, c->stream));
+        }
         const bool fused_y = mc > 0 && pcz && pc_fuse_y;
         if (mc > 0) {
             if (pcz && pc_async) GP2S_TRY(launch_pc_probe(mc, fused_y));
@@ -2733,28 +2863,30 @@ gp2s_status cg_run(gp2s_ctx *c, int m, const V *val, const CGBuffers &B, const d
                                                                     part, pstride);
             else k_update<T><<<nbz, ut, 0, c->stream>>>(n, m, (T *)B.xz, (T *)B.rz, (const T *)B.pz, (const T *)B.qz,
                                                          (T *)B.xy, (T *)B.ry, (const T *)B.py, (const T *)B.qy, sc,
-                                                         part, pstride, nbz);
+                                                         part, pstride, nbz, YFuse(), (const T *)nullptr);
             GP2S_LAUNCH(c);
         }
         if (!fused_y) {
-            if (pcy) GP2S_PCY(PC_UPDATE);
+            if (pcy) GP2S_PCY(PC_UPDATE, fuse);
             else k_update<T><<<nby, ut, 0, c->stream>>>(n, m > 0 ? m : 1, (T *)B.xz, (T *)B.rz, (const T *)B.pz,
                                                          (const T *)B.qz, (T *)B.xy, (T *)B.ry, (const T *)B.py,
-                                                         (const T *)B.qy, sc, part, pstride, 0);
+                                                         (const T *)B.qy, sc, part, pstride, 0, fuse, (const T *)B.py2);
             GP2S_LAUNCH(c);
         }
-        k_scal_beta<<<kc, 256, 0, c->stream>>>(part, part_rr, pstride, fused_y ? (pc_async ? pga : pgz) : pcy ? pgy : nby,
-                                               pcz ? (pc_async ? pga : pgz) : nbz, sc, active, flags + 1, rec, ksteps,
-                                               kmin_probe, pcy, pcz, lucky);
-        GP2S_LAUNCH(c);
-        {
+        if (!fused_scal) {
+            k_scal_beta<<<kc, 256, 0, c->stream>>>(part, part_rr, pstride,
+                                                   fused_y ? (pc_async ? pga : pgz) : pcy ? pgy : nby,
+                                                   pcz ? (pc_async ? pga : pgz) : nbz, sc, active, flags + 1, rec, ksteps,
+                                                   kmin_probe, pcy, pcz, lucky);
+            GP2S_LAUNCH(c);
+        }
+        if (!fuse.dir) {
             // direction: p = z + beta p (z = M^{-1} r for a preconditioned group, z = r otherwise)
             const int cgs = mc / 4;
             const int dthreads = mc > 0 ? cgs * std::max(1, 256 / cgs) : 256;
             const int dgz = mc > 0 ? (int)std::min<int64_t>(152 * 8, ceil_div(n, dthreads / cgs)) : 0;
             const int dgy = (int)std::min<int64_t>(152 * 2, ceil_div(n, dthreads));
             const T *zzp = pcz ? (const T *)B.zz : (const T *)B.rz;
-            const T *zyp = pcy ? (const T *)B.zy : (const T *)B.ry;
             k_direction<T><<<dgz + dgy, dthreads, 0, c->stream>>>(n, mc, zzp, (T *)B.pz, zyp, (T *)B.py, sc, active,
                                                                  dgz, (T *)B.xz, ((pcz && pc_avail) || (!pcz && upd4)) ? 1 : 0);
             GP2S_LAUNCH(c);
@@ -2783,12 +2915,12 @@ gp2s_status cg_run(gp2s_ctx *c, int m, const V *val, const CGBuffers &B, const d
             k_pc_step<PC_REPLACE, 128><<<pgy, kPCThreads, pc_smem(0, 128), c->stream>>>(
                 n, 0, nblky, 0, Minvy, (float *)B.xz, (float *)B.rz, (float *)B.pz, (const float *)B.qz,
                 (float *)B.zz, (float *)B.xy, (float *)B.ry, (float *)B.py, (const float *)B.qy, (float *)B.zy, r64,
-                sc, part, part_rr, pstride, 0);
+                sc, part, part_rr, pstride, 0, YFuse(), nullptr);
         else
             k_pc_step<PC_REPLACE, 64><<<pgy, kPCThreads, pc_smem(0, 64), c->stream>>>(
                 n, 0, nblky, 0, Minvy, (float *)B.xz, (float *)B.rz, (float *)B.pz, (const float *)B.qz,
                 (float *)B.zz, (float *)B.xy, (float *)B.ry, (float *)B.py, (const float *)B.qy, (float *)B.zy, r64,
-                sc, part, part_rr, pstride, 0);
+                sc, part, part_rr, pstride, 0, YFuse(), nullptr);
         GP2S_LAUNCH(c);
         k_scal_replace<<<1, 256, 0, c->stream>>>(part, part_rr, pgy, sc, active, rel->delta);
         GP2S_LAUNCH(c);
@@ -2892,12 +3024,12 @@ gp2s_status y_residual(gp2s_ctx *c, const double *y_sorted_dev, double *relres)
 }
 
 // Layout of the Krylov vectors in c->vec: probe group x, r, p, q (n x m each), y group x, r, p, q
-// (n each), then z of the y column and z of the probe group (block-Jacobi PCG).
+// (n each), then z of the probe group and of the y column (block-Jacobi PCG) and the y group's second p.
 static gp2s_status cg_layout(gp2s_ctx *c, int mm, CGBuffers *B)
 {
     const int64_t n = c->A.n;
     const size_t es = c->A.precision == GP2S_PREC_MIXED ? sizeof(float) : sizeof(double);
-    GP2S_TRY(ensure(c, c->vec, es * (size_t)n * (5 + 5 * (size_t)mm) + 256));
+    GP2S_TRY(ensure(c, c->vec, es * (size_t)n * (6 + 5 * (size_t)mm) + 256));
     char *base = c->vec.as<char>();
     size_t nz = es * (size_t)n * mm;
     B->xz = base; B->rz = base + nz; B->pz = base + 2 * nz; B->qz = base + 3 * nz;
@@ -2905,6 +3037,7 @@ static gp2s_status cg_layout(gp2s_ctx *c, int mm, CGBuffers *B)
     B->xy = yb; B->ry = yb + es * n; B->py = yb + 2 * es * n; B->qy = yb + 3 * es * n;
     B->zz = yb + 4 * es * n;
     B->zy = (char *)B->zz + nz;
+    B->py2 = (char *)B->zy + es * n;
     return GP2S_OK;
 }
 
