@@ -423,6 +423,22 @@ def test_spmm_gather_copies_equal_register_gathers(gp, monkeypatch, probes, n):
         assert i0["spmm_seg_tiles"] > 1
 
 
+@pytest.mark.parametrize("probes,n,row", [(16, 33, 12), (16, 3001, 33), (16, 2500, 120), (48, 1500, 31)])
+def test_fp64_spmm_with_partly_filled_warps(gp, ctx, probes, n, row):
+    """FP64 multi-RHS SpMM where the columns do not fill a warp (16: the half-warps take alternate entries of a
+    row; 48: 24 lanes): rows of odd lengths, beyond one 32-entry batch, a matrix smaller than the grid.
+    Probe solves to 1e-10 on both sides leave about 1e-8 of the gradient."""
+    import oracle
+    w = W.random_small(760 + n, n, 2, L=3, sigma2=1e-2)
+    w["hyper"]["r"] *= (row / 30.0) ** 0.5
+    opts = gp.default_opts(precision=gp.PREC_FP64, logdet=gp.LOGDET_SLQ, probes=probes, lanczos_steps=20, seed=6,
+                           tol_probe=1e-10)
+    lml, g, info = ctx.lml_grad(w["X"], w["y"], gp.Hyper(**w["hyper"]), opts)
+    s = oracle.lml_slq(w["X"], w["y"], oracle.Hyper(**w["hyper"]), m=probes, k=20, seed=6, tol=1e-12)
+    assert info["logdet"] == pytest.approx(s["logdet"], rel=1e-8)
+    assert np.abs(g - s["grad"]).max() <= 1e-7 * np.abs(s["grad"]).max()
+
+
 def test_autograd_function(gp, ctx):
     w = W.random_small(303, 3000, 2, L=2, sigma2=1e-3)
     h = gp.Hyper(**w["hyper"])
