@@ -577,21 +577,27 @@ static gp2s_status far_field_union(gp2s_ctx *c, int64_t n, int L, int64_t *nnz)
     return GP2S_OK;
 }
 
-__global__ void k_rowcnt_minmax(const int32_t *__restrict__ cnt, int64_t n, int *__restrict__ mm)
+// Shortest and longest row, and the largest distance of a stored entry below the diagonal (columns ascend
+// and the diagonal is stored, so a row's first column gives it).
+__global__ void k_rowcnt_minmax(const int32_t *__restrict__ cnt, const int32_t *__restrict__ rowptr,
+                                const int32_t *__restrict__ col, int64_t n, int *__restrict__ mm)
 {
-    int lo = INT32_MAX, hi = 0;
+    int lo = INT32_MAX, hi = 0, band = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         lo = min(lo, cnt[i]);
         hi = max(hi, cnt[i]);
+        band = max(band, (int)i - col[rowptr[i]]);
     }
     for (int o = 16; o > 0; o >>= 1) {
         lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
         hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        band = max(band, __shfl_xor_sync(0xffffffffu, band, o));
     }
     if ((threadIdx.x & 31) == 0) {
         atomicMin(&mm[0], lo);
         atomicMax(&mm[1], hi);
+        atomicMax(&mm[2], band);
     }
 }
 
@@ -1016,14 +1022,14 @@ gp2s_status assemble_problem(gp2s_ctx *c, int64_t n, const double *X_dev, const 
     GP2S_TRY(values_pass(c, n, d, kp, mixed));
     GP2S_CUDA(c, cudaEventRecord(ev[4], c->stream));
     {
-        int init[2] = {INT32_MAX, 0};
+        int init[3] = {INT32_MAX, 0, 0};
         GP2S_CUDA(c, cudaMemcpyAsync(mm, init, sizeof(init), cudaMemcpyHostToDevice, c->stream));
         unsigned gb = (unsigned)std::min<int64_t>(ceil_div(n, 256), 152 * 4);
-        k_rowcnt_minmax<<<gb, 256, 0, c->stream>>>(c->rowcnt.as<int32_t>(), n, mm);
+        k_rowcnt_minmax<<<gb, 256, 0, c->stream>>>(c->rowcnt.as<int32_t>(), c->rowptr.as<int32_t>(), c->col.as<int32_t>(), n, mm);
         GP2S_LAUNCH(c);
     }
     unsigned long long hstats[2];
-    int hmm[2];
+    int hmm[3];
     GP2S_CUDA(c, cudaMemcpyAsync(hstats, stats, sizeof(hstats), cudaMemcpyDeviceToHost, c->stream));
     GP2S_CUDA(c, cudaMemcpyAsync(hmm, mm, sizeof(hmm), cudaMemcpyDeviceToHost, c->stream));
     GP2S_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -1048,6 +1054,7 @@ gp2s_status assemble_problem(gp2s_ctx *c, int64_t n, const double *X_dev, const 
     A.nnz = nnz;
     A.ncells = ncells;
     A.nitems = nitems;
+    A.band = hmm[2];
     A.d = d;
     A.L = L;
     A.precision = o->precision;

@@ -79,6 +79,7 @@ struct Assembled {
     SupportParams sp{};
     gp2s_opts opts{};
     gp2s_assemble_info info{};
+    int band = 0;             // largest distance of a stored entry from the diagonal (sorted numbering)
     double wc_lmax = 0.0;     // Wendland convolution: largest lambda_k over the points (cell edge r sqrt)
 };
 

@@ -439,6 +439,24 @@ def test_fp64_spmm_with_partly_filled_warps(gp, ctx, probes, n, row):
     assert np.abs(g - s["grad"]).max() <= 1e-7 * np.abs(s["grad"]).max()
 
 
+@pytest.mark.parametrize("n,row", [(1, 1), (33, 5), (2049, 150), (20_000, 40), (60_001, 180)])
+def test_band_matrix_y_solve(gp, ctx, n, row):
+    """One-dimensional points in SLQ evaluations without a gradient: y by the tiled Cholesky factor of the
+    band, with the residual of an FP64 solve, and the same evaluation through y's PCG (lml_grad, whose y
+    solve meets 1e-8: its quadratic term agrees to second order in that).  A point, a band as wide as the
+    matrix, rows of several tiles."""
+    w = W.random_small(780 + n, n, 1, L=3, sigma2=1e-3, r=0.05 if n == 1 else None)
+    w["hyper"]["r"] *= row / 30.0
+    h = gp.Hyper(**w["hyper"])
+    opts = gp.default_opts(logdet=gp.LOGDET_SLQ, probes=16, lanczos_steps=min(40, max(1, n // 2)), seed=3)
+    lml, info = ctx.lml(w["X"], w["y"], h, opts)
+    assert info["iters_y"] == 0 and info["relres"] <= 1e-10
+    lml_g, _, info_g = ctx.lml_grad(w["X"], w["y"], h, opts)
+    assert info["quad"] == pytest.approx(info_g["quad"], rel=1e-7)
+    assert info["logdet"] == pytest.approx(info_g["logdet"], rel=1e-6, abs=1e-6)
+    assert ctx.logdet()[0] == pytest.approx(info["logdet"], rel=1e-9, abs=1e-9)
+
+
 def test_autograd_function(gp, ctx):
     w = W.random_small(303, 3000, 2, L=2, sigma2=1e-3)
     h = gp.Hyper(**w["hyper"])
