@@ -85,6 +85,7 @@ gp2s_status batched_lml(gp2s_ctx *c, int32_t B, const int64_t *n, const double *
         // graphs per problem are the autotuner's choice (many host threads capturing at once can
         // cost more than the launches they save on small problems)
         w->use_graphs = false;
+        w->shared_gpu = true;
         c->workers.push_back(w);
         c->worker_streams.push_back(s);
     }

@@ -146,6 +146,7 @@ struct gp2s_ctx {
     std::vector<gp2s_ctx *> workers;
     std::vector<cudaStream_t> worker_streams;
     int batch_workers_max = 16;
+    bool shared_gpu = false;        // a batched worker: other problems run beside this one
     // batched autotuner: per shape class, the summed score (seconds per point) and the number of
     // problems each launch configuration ran, and which configurations were handed out
     struct TuneState {
