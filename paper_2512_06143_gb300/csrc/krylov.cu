@@ -276,7 +276,57 @@ k_spmm(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col, cons
     (void)active;
 }
 
-// CSR SpMV in FP64 (refinement residual): out = b - Ah x.
+// Sums over the warp of four values per lane, one row each, in 6 additions instead of 20 (an FP64
+// instruction costs the SM 19 cycles however few lanes need it): lane masks 16 and 8 also part the rows, so
+// that afterwards lane l holds the sum of value ((l >> 4) & 1) + 2 ((l >> 3) & 1).  Every sum adds the same
+// pairs as warp_sum's tree: the same bits.
+__device__ __forceinline__ double warp_sum4(const double (&s)[4], int lane)
+{
+    const bool hi = (lane & 16) != 0, up = (lane & 8) != 0;
+    const double r01 = (hi ? s[1] : s[0]) + __shfl_xor_sync(0xffffffffu, hi ? s[0] : s[1], 16);
+    const double r23 = (hi ? s[3] : s[2]) + __shfl_xor_sync(0xffffffffu, hi ? s[2] : s[3], 16);
+    double t = (up ? r23 : r01) + __shfl_xor_sync(0xffffffffu, up ? r01 : r23, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
+}
+
+// This lane's parts of rows i0 .. i0 + 3 of A x: 32 entries of each row at a time, the four rows' loads in
+// flight together; a row without entries left pays no FMA.
+__device__ __forceinline__ void dot4_rows(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col,
+                                          const double *__restrict__ val, int64_t n, int64_t i0,
+                                          const double *__restrict__ x, double (&s)[4], int lane)
+{
+    int e[5], most = 0;
+#pragma unroll
+    for (int j = 0; j < 5; ++j) e[j] = rowptr[i0 + j < n ? i0 + j : n];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        s[j] = 0.0;
+        most = max(most, e[j + 1] - e[j]);
+    }
+    for (int o = 0; o < most; o += kWarp) {
+        double v[4], g[4];
+        int cj[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int p = e[j] + o + lane;
+            const bool in = p < e[j + 1];
+            v[j] = in ? __ldcs(val + p) : 0.0;
+            cj[j] = in ? __ldcs(col + p) : -1;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) g[j] = cj[j] >= 0 ? x[cj[j]] : 0.0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (e[j] + o < e[j + 1]) s[j] = cj[j] >= 0 ? fma(v[j], g[j], s[j]) : s[j];
+    }
+}
+
+// CSR SpMV in FP64 (refinement residual): out = b - Ah x, four consecutive rows per warp at a time.
+// Bounded by the FP64 pipe before HBM (12 bytes per entry): per row of up to 64 entries 2 FMAs and, shared
+// by four rows, 6 additions; a tree of 5 additions per row took 5.4 ms at N = 10M
+// (4.3 scaled to 8M); now 2.04 ms at N = 8M, 491 M entries, 2.9 TB/s.
 __global__ void __launch_bounds__(256)
 k_residual64(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col,
              const double *__restrict__ val, int64_t n, const double *__restrict__ x,
@@ -285,11 +335,13 @@ k_residual64(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col
     const int lane = threadIdx.x & 31;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t i = w0; i < n; i += nw) {
-        double s = 0.0;
-        for (int p = rowptr[i] + lane; p < rowptr[i + 1]; p += kWarp) s = fma(__ldcs(val + p), x[__ldcs(col + p)], s);
-        s = warp_sum(s);
-        if (lane == 0) out[i] = b[i] - s;
+    const int mine = ((lane >> 4) & 1) + 2 * ((lane >> 3) & 1);   // the row whose sum this lane gets
+    for (int64_t i0 = w0 * 4; i0 < n; i0 += nw * 4) {
+        double s[4];
+        dot4_rows(rowptr, col, val, n, i0, x, s, lane);
+        const double t = warp_sum4(s, lane);
+        const int64_t i = i0 + mine;
+        if ((lane & 7) == 0 && i < n) out[i] = b[i] - t;
     }
 }
 
@@ -864,6 +916,46 @@ k_spmv_y(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col, co
     }
 }
 
+// The FP64 form: bounded by the FP64 pipe (two FMAs per row of up to 64 entries, the tree, the dot), so
+// four consecutive rows share their trees (warp_sum4), the dot takes one FMA for the four, and a row pays
+// only for the 32-entry pieces that it has.  LML and gradient at 30,011 points 39.2 -> 34.5 ms.
+__global__ void __launch_bounds__(kSpmvThreads)
+k_spmv_y64(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col, const double *__restrict__ val, int64_t n,
+           const double *__restrict__ py, double *__restrict__ qy, double *__restrict__ part, YFuse f)
+{
+    __shared__ double sh[kSpmvThreads / kWarp];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int mine = ((lane >> 4) & 1) + 2 * ((lane >> 3) & 1);   // the row whose sum this lane gets
+    double d = 0.0;
+    for (int64_t i0 = w0 * 4; i0 < n; i0 += nw * 4) {
+        double s[4];
+        dot4_rows(rowptr, col, val, n, i0, py, s, lane);
+        const double t = warp_sum4(s, lane);
+        const int64_t i = i0 + mine;
+        const bool own = (lane & 7) == 0 && i < n;
+        if (own) qy[i] = t;
+        d = fma(own ? py[i] : 0.0, t, d);
+    }
+    d = warp_sum(d);
+    if (lane == 0) sh[wid] = d;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int w = 0; w < kSpmvThreads / kWarp; ++w) t += sh[w];
+        part[blockIdx.x] = t;
+    }
+    if (f.sc && last_cta(&f.flags[4], gridDim.x)) {
+        const double s = block_sum(part, gridDim.x);
+        if (threadIdx.x == 0) {
+            f.flags[4] = 0;
+            f.flags[1] = f.flags[2] = 0;
+            scal_alpha(0, s, f.sc, f.active, f.flags, nullptr, 0, f.lucky);
+        }
+    }
+}
+
 // The FP32 multi-RHS SpMM runs on the RB8 copy when it has been built.
 template <class T>
 bool rb_launch(gp2s_ctx *c, int m, bool has_y)
@@ -959,7 +1051,9 @@ gp2s_status launch_spmm(gp2s_ctx *c, int m, bool has_y, const V *val, const CGBu
         const int nbv = (int)std::min<int64_t>(std::min(kSpmvBlocks, pstride),
                                                std::max<int64_t>(1, ceil_div(A.n * kWarp, kSpmvThreads)));
         T *pa = (T *)B.py, *pb = (T *)B.py2;
-        if (fuse.dir) k_spmv_y<T, V, true><<<nbv, kSpmvThreads, 0, c->stream>>>(rp, cl, val, A.n, pa, pb, zy, qy, part, fuse);
+        if constexpr (std::is_same<T, double>::value)
+            k_spmv_y64<<<nbv, kSpmvThreads, 0, c->stream>>>(rp, cl, val, A.n, pa, qy, part, fuse);
+        else if (fuse.dir) k_spmv_y<T, V, true><<<nbv, kSpmvThreads, 0, c->stream>>>(rp, cl, val, A.n, pa, pb, zy, qy, part, fuse);
         else k_spmv_y<T, V, false><<<nbv, kSpmvThreads, 0, c->stream>>>(rp, cl, val, A.n, pa, pb, zy, qy, part, fuse);
         GP2S_LAUNCH(c);
         *nparts = nbv;
@@ -2864,7 +2958,9 @@ gp2s_status cg_run(gp2s_ctx *c, int m, const V *val, const CGBuffers &B, const d
             fuse.active = active;
             fuse.flags = flags;
             fuse.lucky = lucky;
-            fuse.dir = n <= kYDirRows && !rel;   // a residual replacement continues from p in its own buffer
+            // (a residual replacement continues from p in its own buffer; in FP64 the second FMA per entry
+            // costs more than the launch)
+            fuse.dir = n <= kYDirRows && !rel && std::is_same<T, float>::value;
         }
         GP2S_TRY((launch_spmm<T, V>(c, mc, true, val, B, part, pstride, nb, rsplit, active, &np, dev_err, fuse, zyp)));
         if (!fused_scal) {
