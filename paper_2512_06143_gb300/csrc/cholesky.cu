@@ -13,9 +13,9 @@
 // short (its length per tile column falls with the tile's size squared), and the ordering prefers
 // tile columns that do not wait on others (a band of 63 tile columns becomes a chain of 11).  One kernel
 // with a flag per tile takes the place of four launches per panel of the whole matrix.
-// Measured: the FP64 LML of 4,096 points in 2-D 52.1 -> 3.2 ms (this kernel 2.4), an MCMC evaluation of
-// 2,000 points in 1-D 18.4 -> 0.71 ms (0.51), the allocation-free call at 301 points, all tiles
-// present, 2.47 -> 0.45 ms.
+// Measured: the FP64 LML of 4,096 points in 2-D 52.1 -> 3.16 ms, an MCMC evaluation of 2,000 points in 1-D
+// 18.4 -> 0.74 ms, the allocation-free call at 301 points, all tiles present, 2.47 -> 0.45 ms; with the pivots'
+// tests and reciprocals mostly off the FP64 pipe 2.74, 0.70 and 0.41 ms.
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -53,13 +53,25 @@ __device__ __forceinline__ bool chol_wait(const int *flag, const int *abort_word
     return false;
 }
 
-// 1 / d for a positive normal d: the FP32 reciprocal (relative error e below 2^-21) and one cubic
-// step r (1 + e + e^2), three dependent FP64 operations instead of a full division's chain (an
-// FP64 operation takes 64 cycles here); out of FP32's comfortable range the division itself.
+// A pivot d is usable when its sign bit is clear and it is neither zero, infinite nor NaN: read off its high
+// word, since an FP64 comparison takes as long as an FP64 addition (64 cycles of the warp).
+__device__ __forceinline__ bool chol_positive(double d)
+{
+    const int hi = __double2hiint(d);
+    return hi < 0x7ff00000 && (hi > 0 || (hi == 0 && __double2loint(d) != 0));
+}
+
+// 1 / d for a usable pivot: the FP32 reciprocal (relative error e below 2^-20) and one cubic step
+// r (1 + e + e^2), three dependent FP64 operations instead of a full division's chain.  The conversions
+// to FP32 and back move the exponent and the upper 23 bits of the mantissa with integer operations, as
+// converting is FP64 work too; outside 2^-100 .. 2^100 the division itself.
 __device__ __forceinline__ double chol_rcp(double d)
 {
-    if (!(d > 1e-30 && d < 1e30)) return 1.0 / d;
-    const double r = (double)(1.0f / (float)d);
+    const int hi = __double2hiint(d), lo = __double2loint(d);
+    if (hi < ((1023 - 100) << 20) || hi >= ((1023 + 100) << 20)) return 1.0 / d;
+    const float f = __int_as_float(((hi - ((1023 - 127) << 20)) << 3) | (int)((unsigned)lo >> 29));
+    const int rf = __float_as_int(1.0f / f);
+    const double r = __hiloint2double((rf >> 3) + ((1023 - 127) << 20), rf << 29);
     const double e = fma(-d, r, 1.0);
     return fma(r, fma(e, e, e), r);
 }
@@ -278,7 +290,7 @@ k_chol(const CholArgs a)
                     // rows up to c are finished (a warp holds eight rows)
                     if (8 * wid + 7 > c) {
                         double d = colbuf[c & 1][c];
-                        if (!(d > 0.0)) d = 1.0;
+                        if (!chol_positive(d)) d = 1.0;
                         const double w = colbuf[c & 1][r4] * chol_rcp(d);
 #pragma unroll
                         for (int m = 0; m < 8; ++m)
