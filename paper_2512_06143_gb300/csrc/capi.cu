@@ -419,7 +419,7 @@ gp2s_status gp2s_logdet(gp2s_ctx *c, double *logdet, double *stderr_hat, gp2s_lo
         GP2S_TRY(ensure(c, c->ys64, sizeof(double) * A.n));
         GP2S_CUDA(c, cudaMemsetAsync(c->ys64.p, 0, sizeof(double) * A.n, c->stream));
         CGResult res;
-        gp2s_status st = krylov_solve(c, c->ys64.as<double>(), true, m, A.opts.lanczos_steps, &res);
+        gp2s_status st = krylov_solve(c, c->ys64.as<double>(), true, m, A.opts.lanczos_steps, &res, true);
         if (st != GP2S_OK && st != GP2S_ENOCONV) return st;
         c->have_solution = false;
         GP2S_TRY(slq_logdet(c, m, A.opts.lanczos_steps, &lhat, &se));

@@ -248,8 +248,9 @@ struct CGResult {
     double relres = 0.0;
     gp2s_status status = GP2S_OK;
 };
+// y_zero: y_sorted_dev is known to be all zeros (the y column stays idle).
 gp2s_status krylov_solve(gp2s_ctx *c, const double *y_sorted_dev, bool with_probes, int m,
-                         int ksteps, CGResult *res);
+                         int ksteps, CGResult *res, bool y_zero = false);
 gp2s_status slq_logdet(gp2s_ctx *c, int m, int ksteps, double *logdet_hat, double *stderr_hat);
 // Start SLQ's quadratures on the side stream from the coefficients recorded so far (every probe
 // column has its k steps or has stopped); the stream order of c->stream is the dependency.

@@ -822,7 +822,7 @@ struct CGBuffers {
 };
 
 template <int KH, int NG>
-gp2s_status launch_rb(gp2s_ctx *c, const CGBuffers &B, double *part, int pstride, int nb, int *nparts);
+gp2s_status launch_rb(gp2s_ctx *c, const CGBuffers &B, double *part, int pstride, int nb, int *nparts, bool has_y);
 template <int NG>
 gp2s_status launch_rb4_et(gp2s_ctx *c, const CGBuffers &B, double *part, int pstride, int nb, int *nparts, int *err,
                           int et, bool *done);
@@ -958,9 +958,9 @@ k_spmv_y64(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col, 
 
 // The FP32 multi-RHS SpMM runs on the RB8 copy when it has been built.
 template <class T>
-bool rb_launch(gp2s_ctx *c, int m, bool has_y)
+bool rb_launch(gp2s_ctx *c, int m)
 {
-    return std::is_same<T, float>::value && c->rb_valid && m > 0 && has_y;
+    return std::is_same<T, float>::value && c->rb_valid && m > 0;
 }
 
 // Row ranges of the SpMM CTAs with equal shares of the entries: split[b] = first row whose entries
@@ -1016,7 +1016,7 @@ gp2s_status launch_spmm(gp2s_ctx *c, int m, bool has_y, const V *val, const CGBu
         c->prof_used += 2;
         GP2S_CUDA(c, cudaEventRecord(ev_a, c->stream));
     }
-    if (rb_launch<T>(c, m, has_y)) {
+    if (rb_launch<T>(c, m)) {
         // 16, 32 and 64 columns can take the gather-copy form (ET copied rows per 32-entry batch)
         bool done = false;
         if (c->spmm_tma > 0 && !c->spmm_half) {
@@ -1032,17 +1032,17 @@ gp2s_status launch_spmm(gp2s_ctx *c, int m, bool has_y, const V *val, const CGBu
         // every lane covers KH = 4 columns where the column count allows (groups of 4, 8 or 16
         // lanes per entry); 48 and 96 columns take half-warps with KH = 3 and 6
         case 16:
-            GP2S_TRY((c->spmm_half ? launch_rb<1, 2>(c, B, part, pstride, nb, nparts)
-                                   : launch_rb<4, 8>(c, B, part, pstride, nb, nparts)));
+            GP2S_TRY((c->spmm_half ? launch_rb<1, 2>(c, B, part, pstride, nb, nparts, has_y)
+                                   : launch_rb<4, 8>(c, B, part, pstride, nb, nparts, has_y)));
             break;
         case 32:
-            GP2S_TRY((c->spmm_half ? launch_rb<2, 2>(c, B, part, pstride, nb, nparts)
-                                   : launch_rb<4, 4>(c, B, part, pstride, nb, nparts)));
+            GP2S_TRY((c->spmm_half ? launch_rb<2, 2>(c, B, part, pstride, nb, nparts, has_y)
+                                   : launch_rb<4, 4>(c, B, part, pstride, nb, nparts, has_y)));
             break;
-        case 48: GP2S_TRY((launch_rb<3, 2>(c, B, part, pstride, nb, nparts))); break;
-        case 64: GP2S_TRY((launch_rb<4, 2>(c, B, part, pstride, nb, nparts))); break;
-        case 96: GP2S_TRY((launch_rb<6, 2>(c, B, part, pstride, nb, nparts))); break;
-        default: GP2S_TRY((launch_rb<8, 2>(c, B, part, pstride, nb, nparts))); break;
+        case 48: GP2S_TRY((launch_rb<3, 2>(c, B, part, pstride, nb, nparts, has_y))); break;
+        case 64: GP2S_TRY((launch_rb<4, 2>(c, B, part, pstride, nb, nparts, has_y))); break;
+        case 96: GP2S_TRY((launch_rb<6, 2>(c, B, part, pstride, nb, nparts, has_y))); break;
+        default: GP2S_TRY((launch_rb<8, 2>(c, B, part, pstride, nb, nparts, has_y))); break;
         }
         if (ev_b) GP2S_CUDA(c, cudaEventRecord(ev_b, c->stream));
         return GP2S_OK;
@@ -1855,11 +1855,11 @@ inline RBTiles rb_tiles(int64_t nblk, int nb, bool shared_gpu)
 }
 
 template <int KH, int NG>
-gp2s_status launch_rb(gp2s_ctx *c, const CGBuffers &B, double *part, int pstride, int nb, int *nparts)
+gp2s_status launch_rb(gp2s_ctx *c, const CGBuffers &B, double *part, int pstride, int nb, int *nparts, bool has_y)
 {
     constexpr int M = kWarp / NG * KH;
     const size_t smem = rb_smem<KH>();
-    auto kern = k_spmm_rb<KH, NG, true>;
+    auto kern = has_y ? k_spmm_rb<KH, NG, true> : k_spmm_rb<KH, NG, false>;
     GP2S_TRY(smem_attr(c, (const void *)kern, smem));
     const RBTiles tl = rb_tiles(ceil_div(c->A.n, kRB), nb, c->shared_gpu);
     GP2S_TRY(ensure(c, c->rb_tpart, sizeof(double) * (size_t)tl.ntiles * (M + 1)));
@@ -2785,10 +2785,13 @@ struct ReliableY {
 };
 
 // One CG run (x0 = 0) on columns [y | probes]; the probe right-hand sides must already be in rz.
+// y_idle: rhs_y is zero, so the y column is inactive from the start and its part of every step is left out
+// (a log-determinant of 200,003 points in 2-D 26.3 -> 23.5 ms, a posterior variance of 200 points on 100,000
+// 73.8 -> 64 ms).
 template <class T, class V>
 gp2s_status cg_run(gp2s_ctx *c, int m, const V *val, const CGBuffers &B, const double *rhs_y, double tol_y,
                    double tol_z, int kmin_probe, int ksteps, double *rec, int max_iter, int *iters_y,
-                   int *iters_z, bool *breakdown, ReliableY *ru = nullptr)
+                   int *iters_z, bool *breakdown, ReliableY *ru = nullptr, bool y_idle = false)
 {
     const Assembled &A = c->A;
     const int64_t n = A.n;
@@ -2962,13 +2965,13 @@ gp2s_status cg_run(gp2s_ctx *c, int m, const V *val, const CGBuffers &B, const d
             // costs more than the launch)
             fuse.dir = n <= kYDirRows && !rel && std::is_same<T, float>::value;
         }
-        GP2S_TRY((launch_spmm<T, V>(c, mc, true, val, B, part, pstride, nb, rsplit, active, &np, dev_err, fuse, zyp)));
+        GP2S_TRY((launch_spmm<T, V>(c, mc, !y_idle || mc == 0, val, B, part, pstride, nb, rsplit, active, &np, dev_err, fuse, zyp)));
         if (!fused_scal) {
             k_scal_alpha<<<kc, 256, 0, c->stream>>>(part, pstride, np, sc, active, flags, rec, ksteps, lucky);
             GP2S_LAUNCH(c);
             GP2S_CUDA(c, cudaMemsetAsync(flags + 1, 0, sizeof(int) * 2, c->stream));
         }
-        const bool fused_y = mc > 0 && pcz && pc_fuse_y;
+        const bool fused_y = mc > 0 && pcz && pc_fuse_y && !y_idle;
         if (mc > 0) {
             if (pcz && pc_async) GP2S_TRY(launch_pc_probe(mc, fused_y));
             else if (pcz) GP2S_PCZ_WY(PC_UPDATE, mc, fused_y ? 1 : 0);
@@ -2979,7 +2982,7 @@ gp2s_status cg_run(gp2s_ctx *c, int m, const V *val, const CGBuffers &B, const d
                                                          part, pstride, nbz, YFuse(), (const T *)nullptr);
             GP2S_LAUNCH(c);
         }
-        if (!fused_y) {
+        if (!fused_y && (!y_idle || mc == 0)) {
             if (pcy) GP2S_PCY(PC_UPDATE, fuse);
             else k_update<T><<<nby, ut, 0, c->stream>>>(n, m > 0 ? m : 1, (T *)B.xz, (T *)B.rz, (const T *)B.pz,
                                                          (const T *)B.qz, (T *)B.xy, (T *)B.ry, (const T *)B.py,
@@ -3181,10 +3184,10 @@ gp2s_status krylov_columns_solve(gp2s_ctx *c, int m, double tol, int *iters)
     bool brk = false;
     if (mixed)
         GP2S_TRY((cg_run<float, float>(c, m, c->val32.as<float>(), B, zero, 1.0, tol, 0, 0, nullptr, A.opts.max_iter,
-                                       &iy, &iz, &brk)));
+                                       &iy, &iz, &brk, nullptr, true)));
     else
         GP2S_TRY((cg_run<double, double>(c, m, c->val64.as<double>(), B, zero, 1.0, tol, 0, 0, nullptr,
-                                         A.opts.max_iter, &iy, &iz, &brk)));
+                                         A.opts.max_iter, &iy, &iz, &brk, nullptr, true)));
     c->have_probes = false;
     *iters = iz;
     if (brk) return set_err(c, GP2S_EBREAKDOWN, "CG breakdown in a posterior-variance solve");
@@ -3206,7 +3209,7 @@ static bool y_direct(const gp2s_ctx *c)
 }
 
 gp2s_status krylov_solve(gp2s_ctx *c, const double *y_sorted_dev, bool with_probes, int m, int ksteps,
-                         CGResult *res)
+                         CGResult *res, bool y_zero)
 {
     Assembled &A = c->A;
     const int64_t n = A.n;
@@ -3254,10 +3257,10 @@ gp2s_status krylov_solve(gp2s_ctx *c, const double *y_sorted_dev, bool with_prob
             GP2S_CUDA(c, cudaMemsetAsync(r64, 0, sizeof(double) * n, c->stream));
             if (mixed)
                 GP2S_TRY((cg_run<float, float>(c, mm, c->val32.as<float>(), B, r64, 1.0, tol_z, ksteps, ksteps, rec,
-                                               o.max_iter, &iy, &iz, &brk)));
+                                               o.max_iter, &iy, &iz, &brk, nullptr, true)));
             else
                 GP2S_TRY((cg_run<double, double>(c, mm, c->val64.as<double>(), B, r64, 1.0, tol_z, ksteps, ksteps, rec,
-                                                 o.max_iter, &iy, &iz, &brk)));
+                                                 o.max_iter, &iy, &iz, &brk, nullptr, true)));
             if (brk) return set_err(c, GP2S_EBREAKDOWN, "CG breakdown in a probe column");
         }
         // ... and the y column is MINRES's: FP64 on Ah, restarted on the FP64 residual
@@ -3295,11 +3298,11 @@ gp2s_status krylov_solve(gp2s_ctx *c, const double *y_sorted_dev, bool with_prob
     // an evaluation without a gradient (training, batches) on a band matrix: the probe columns run their
     // Lanczos steps beside an idle y column, and y is solved by the tiled Cholesky factor; where that fails
     // the y column's PCG follows on its own
-    const bool direct = mixed && mm > 0 && !c->probes_for_grad && o.precond == 2 && y_direct(c);
+    const bool direct = mixed && mm > 0 && !y_zero && !c->probes_for_grad && o.precond == 2 && y_direct(c);
     if (direct) {
         GP2S_CUDA(c, cudaMemsetAsync(r64, 0, sizeof(double) * n, c->stream));
         GP2S_TRY((cg_run<float, float>(c, mm, c->val32.as<float>(), B, r64, 1.0, tol_z, ksteps, ksteps, rec, o.max_iter,
-                                       &iy, &iz, &brk)));
+                                       &iy, &iz, &brk, nullptr, true)));
         if (brk) return set_err(c, GP2S_EBREAKDOWN, "CG breakdown (p^T A p <= 0 or NaN)");
         double ld = 0.0, relres = 0.0;
         const gp2s_status st = exact_logdet_solve(c, y_sorted_dev, &ld);
@@ -3333,14 +3336,14 @@ gp2s_status krylov_solve(gp2s_ctx *c, const double *y_sorted_dev, bool with_prob
     // about ten launches and up to one check interval of idle y iterations, which a small problem's
     // cheap restarted refinement undercuts (the 256-problem batch, n <= 65,536: 21 problems/s with
     // them against 29 without; at n = 1M and 10M they save 13 % and 10 %).
-    const bool reliable = c->reliable_y && n >= c->reliable_min_rows;
+    const bool reliable = c->reliable_y && n >= c->reliable_min_rows && !y_zero;
     if (mixed)
         GP2S_TRY((cg_run<float, float>(c, my, c->val32.as<float>(), B, b64, tol_first, tol_z, my > 0 ? ksteps : 0,
                                        ksteps, my > 0 ? rec : nullptr, o.max_iter, &iy, &iz, &brk,
-                                       reliable ? &ru : nullptr)));
+                                       reliable ? &ru : nullptr, y_zero)));
     else
         GP2S_TRY((cg_run<double, double>(c, mm, c->val64.as<double>(), B, b64, tol_first, tol_z,
-                                         mm > 0 ? ksteps : 0, ksteps, rec, o.max_iter, &iy, &iz, &brk)));
+                                         mm > 0 ? ksteps : 0, ksteps, rec, o.max_iter, &iy, &iz, &brk, nullptr, y_zero)));
     if (!direct) res->iters_probes = iz;
     int total_y = iy;
     if (brk) {
@@ -3355,7 +3358,7 @@ gp2s_status krylov_solve(gp2s_ctx *c, const double *y_sorted_dev, bool with_prob
     // refinement: r = b - Ah xhat in FP64; original-space residual |r / s| / |y|
     double relres = 0.0;
     int outer = 0;
-    for (;;) {
+    while (!y_zero) {
         GP2S_TRY(y_residual(c, y_sorted_dev, &relres));
         if (!(relres > o.tol_refine) || outer >= o.max_outer) break;
         ++outer;
