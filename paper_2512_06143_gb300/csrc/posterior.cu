@@ -13,6 +13,7 @@
 //     k^T A^{-1} k  ~=  2 (s k)^T v - v^T Ah v        (Ah with its FP64 values),
 // the Galerkin (energy) form: its error is -e^T Ah e for the solution error e, second order in the
 // solve's accuracy whatever the precision the solve ran in.
+#include <climits>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -238,7 +239,11 @@ k_post_rhs(PostArgs a, GridParams g, KernelParams kp, int64_t t0, int nb, int m,
 // Column quadratic forms x_c^T Ah x_c of the n x m solution block in FP64 (FP64 values, the
 // stored x taken as exact): one warp per row, lane l owns columns l, l + 32 (m <= 64); per-CTA
 // partials in part[c * gridDim.x + block].
-template <class T>
+// Bounded by the FP64 pipe (a conversion and an FMA per entry and 32 columns, 19 cycles of the SM each), so only
+// the entries below the diagonal are visited: x^T A x = sum_i x_i (2 sum_{j<i} A_ij x_j + A_ii x_i),
+// columns ascending.  All entries, one at a time: 2.12 ms for 64 columns at 100,000 rows of 80 entries, a tenth
+// of the variance of 200 points there (64 -> 61 ms with this).
+template <class T, bool TWO>
 __global__ void __launch_bounds__(kPostThreads)
 k_post_xax(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col, const double *__restrict__ val,
            int64_t n, int m, const T *__restrict__ x, double *__restrict__ part)
@@ -248,20 +253,38 @@ k_post_xax(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col, 
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     double acc0 = 0.0, acc1 = 0.0;
-    const bool c1 = lane + 32 < m;
     for (int64_t i = w0; i < n; i += nw) {
         double s0 = 0.0, s1 = 0.0;
-        for (int p = rowptr[i]; p < rowptr[i + 1]; ++p) {
-            const int j = col[p];
-            const double v = val[p];
-            s0 = fma(v, (double)x[(int64_t)j * m + lane], s0);
-            if (c1) s1 = fma(v, (double)x[(int64_t)j * m + lane + 32], s1);
+        const int p1 = rowptr[i + 1];
+        int p = rowptr[i];
+        // 32 entries at a time, one per lane; the warp goes through those left of the diagonal
+        for (; p < p1; p += 32) {
+            const bool in = p + lane < p1;
+            const int cl = in ? col[p + lane] : INT_MAX;
+            const double vl = in ? val[p + lane] : 0.0;
+            const int left = __popc(__ballot_sync(0xffffffffu, cl < (int)i));
+#pragma unroll 4
+            for (int t = 0; t < left; ++t) {
+                const int64_t j = __shfl_sync(0xffffffffu, cl, t);
+                const double v = __shfl_sync(0xffffffffu, vl, t);
+                s0 = fma(v, (double)x[j * m + lane], s0);
+                if (TWO) s1 = fma(v, (double)x[j * m + lane + 32], s1);
+            }
+            if (left < 32) {
+                // the diagonal follows in this batch
+                const double d = __shfl_sync(0xffffffffu, vl, left);
+                const double x0 = (double)x[i * m + lane];
+                acc0 = fma(x0, fma(d, x0, s0 + s0), acc0);
+                if (TWO) {
+                    const double x1 = (double)x[i * m + lane + 32];
+                    acc1 = fma(x1, fma(d, x1, s1 + s1), acc1);
+                }
+                break;
+            }
         }
-        acc0 = fma((double)x[i * m + lane], s0, acc0);
-        if (c1) acc1 = fma((double)x[i * m + lane + 32], s1, acc1);
     }
     sh[wid][lane] = acc0;
-    if (m > 32) sh[wid][lane + 32] = acc1;
+    if (TWO) sh[wid][lane + 32] = acc1;
     __syncthreads();
     if ((int)threadIdx.x < m) {
         double t = 0.0;
@@ -333,12 +356,12 @@ gp2s_status posterior_d(gp2s_ctx *c, const PostArgs &pa, double *mean_dev, doubl
             ++batches;
             const int nbk = (int)std::min<int64_t>(ceil_div(n, kPostThreads / 32), nblk);
             const int32_t *rp = c->rowptr.as<int32_t>(), *cl = c->col.as<int32_t>();
-            if (mixed)
-                k_post_xax<float><<<nbk, kPostThreads, 0, c->stream>>>(rp, cl, c->val64.as<double>(), n, m,
-                                                                       (const float *)xz, c->post_part.as<double>());
-            else
-                k_post_xax<double><<<nbk, kPostThreads, 0, c->stream>>>(rp, cl, c->val64.as<double>(), n, m,
-                                                                        (const double *)xz, c->post_part.as<double>());
+            const double *v64 = c->val64.as<double>();
+            double *xp = c->post_part.as<double>();
+            if (mixed && m > 32) k_post_xax<float, true><<<nbk, kPostThreads, 0, c->stream>>>(rp, cl, v64, n, m, (const float *)xz, xp);
+            else if (mixed) k_post_xax<float, false><<<nbk, kPostThreads, 0, c->stream>>>(rp, cl, v64, n, m, (const float *)xz, xp);
+            else if (m > 32) k_post_xax<double, true><<<nbk, kPostThreads, 0, c->stream>>>(rp, cl, v64, n, m, (const double *)xz, xp);
+            else k_post_xax<double, false><<<nbk, kPostThreads, 0, c->stream>>>(rp, cl, v64, n, m, (const double *)xz, xp);
             GP2S_LAUNCH(c);
             if (mixed)
                 k_post_var<D, float><<<gb, kPostThreads, 0, c->stream>>>(pa, A.gp, A.kp, t0, nb, m, (const float *)xz,
