@@ -13,8 +13,15 @@ namespace gp2s {
 template <class T>
 __device__ __forceinline__ T wendland(int kind, int d, T t)
 {
-    if (!(t < T(1))) return T(0);
-    if (t < T(0)) t = T(0);
+    if constexpr (sizeof(T) == 8) {
+        // read off the high word: an FP64 comparison costs as much as an addition
+        const int hi = __double2hiint((double)t);
+        if (hi >= 0x3ff00000) return T(0);
+        if (hi < 0) t = T(0);
+    } else {
+        if (!(t < T(1))) return T(0);
+        if (t < T(0)) t = T(0);
+    }
     const T u = T(1) - t;
     const T u2 = u * u;
     if (kind == 1) {
@@ -56,5 +63,26 @@ __device__ __forceinline__ T wendland_dt_over_t(int kind, int d, T t)
     if (d <= 3) return T(-20) * (u2 * u);
     return T(-30) * (u2 * u2);
 }
+
+#ifdef __CUDACC__
+// Square root of q >= 0 in six FP64 operations: the FP32 reciprocal root y of q (its exponent and upper
+// mantissa bits moved to FP32 and back by integer operations, since conversions are FP64 work), one coupled
+// Newton step for g ~ sqrt(q) and h ~ 1 / (2 sqrt(q)) (Goldschmidt's iteration), and the residual
+// correction g + (q - g^2) h, whose own error is below 2^-80 relative: the rounding of the last
+// operation remains.  Zero, and values outside 2^-100 .. 2^100, take sqrt().
+__device__ __forceinline__ double sqrt_pos(double q)
+{
+    const int hi = __double2hiint(q), lo = __double2loint(q);
+    if (hi < ((1023 - 100) << 20) || hi >= ((1023 + 100) << 20)) return sqrt(q);
+    const float f = __int_as_float(((hi - ((1023 - 127) << 20)) << 3) | (int)((unsigned)lo >> 29));
+    const int yb = __float_as_int(rsqrtf(f));
+    const int yhi = (yb >> 3) + ((1023 - 127) << 20);
+    const double y = __hiloint2double(yhi, yb << 29), h0 = __hiloint2double(yhi - (1 << 20), yb << 29);
+    const double g0 = q * y;
+    const double e = fma(-g0, h0, 0.5);
+    const double g = fma(g0, e, g0), h = fma(h0, e, h0);
+    return fma(fma(-g, g, q), h, g);
+}
+#endif
 
 }  // namespace gp2s
