@@ -2319,57 +2319,69 @@ k_pc_step(int64_t n, int m, int64_t nblk, int gz, const float *__restrict__ Minv
 // next block is prefetched into registers.  Every wait on a stage's mbarrier is bounded: after
 // about a second without the copy completing the kernel sets err and returns.
 // ---------------------------------------------------------------------------------------------
-constexpr int kPPThreads = 512;
+constexpr int kPPProducers = 256, kPPConsumers = 128;
+constexpr int kPPThreads = kPPProducers + kPPConsumers;
+// CTAs per SM: 64-row blocks and 32 columns leave room for two (101 KB of stages each)
+template <int SB, int M> constexpr int pp_ctas = (SB == 64 && M == 32) ? 2 : 1;
 
-// two stages of (M^{-1} block, residual block), the y column's two staged residual blocks and its
-// split products (WY), the two mbarriers
+// two stages of (M^{-1} block, residual block), the y column's two staged residual blocks (WY), the
+// two mbarriers
 template <int BJ, int SB, int M>
 size_t pp_smem()
 {
-    return sizeof(float) * (2 * ((size_t)BJ * SB + (size_t)BJ * M) + 2 * (size_t)BJ + 4 * (size_t)BJ) + 64;
+    return sizeof(float) * (2 * ((size_t)BJ * SB + (size_t)BJ * M) + 2 * (size_t)BJ) + 64;
 }
 
 // WY: the y column's PCG update rides along on the same staged M^{-1} blocks (when it uses the
 // probes' factors): x_y += alpha_y p_y, r_y -= alpha_y q_y by the producers, z_y = M^{-1} r_y by the
-// consumers (each half of them sums half of the block's columns), partial dots in column 0 of
+// consumers (one row each, the block's halves summed apart), partial dots in column 0 of
 // part_rz / part_rr.  This saves the y column's own pass over all of M^{-1} per iteration.
 // Stages of BJ = 128 rows; the block-Jacobi blocks are SB = 128 or 64 rows (a stage then holds two
 // consecutive 64 x 64 blocks of M^{-1}, contiguous in memory, and each tile multiplies within its
 // own block).
 template <int BJ, int SB, int M, bool WY>
-__global__ void __launch_bounds__(kPPThreads, 1)
+__global__ void __launch_bounds__(kPPThreads, (pp_ctas<SB, M>))
 k_pc_probe(int64_t n, int64_t nblk, const float *__restrict__ Minv32, float *__restrict__ rz,
            const float *__restrict__ qz, float *__restrict__ zz, const double *__restrict__ sc,
            double *__restrict__ part_rz, double *__restrict__ part_rr, int pstride, int *__restrict__ err,
            float *__restrict__ xy, float *__restrict__ ry, const float *__restrict__ py, const float *__restrict__ qy,
            float *__restrict__ zy)
 {
-    // Warp-specialised: warps 8..15 (producers) turn the staged r of block k into r - alpha q and
-    // hand the stage over through named barrier 1 + (k & 1); warps 0..7 (consumers) take it, form
-    // z = M^{-1} r with 8 x 4 register tiles (one tile per thread), then release the stage, and
+    // Warp-specialised: warps 4..11 (producers) turn the staged r of block k into r - alpha q and
+    // hand the stage over through named barrier 1 + (k & 1); warps 0..3 (consumers) take it, form
+    // z = M^{-1} r with one register tile per thread, then release the stage, and
     // thread 0 refills it with block k + 2.  The producers' elementwise work of block k + 1
     // overlaps the consumers' product of block k.
-    constexpr int NT = kPPThreads / 2;         // threads per role
-    constexpr int CG = M / 4;                  // column groups of four
+    // A consumer's tile is 8 rows x 8 columns with 64 columns (4 loads of 16 bytes for 32 packed FMAs; 8 x 4
+    // tiles of twice the threads took 3 for 16, and shared-memory loads and FMAs of this size do not
+    // overlap: their times added up), 8 x 4 with 32.  The 8 columns are two runs of 4, M / 2 apart, so that
+    // the lanes' loads stay contiguous.  (Scalar FMAs in place of the packed ones: 446 against 402 us at 1M rows.)
+    // Per launch, 64-row blocks at 100,000 rows: 64 columns 49.9 us with 8 x 4 tiles and the y column, 32.8
+    // without y; 32 columns with y 40.4 -> 28.6 (two CTAs per SM, the y column's sums by trees).
+    // 128-row blocks at 1M rows: 403 us before and after, bound by the consumers' FMAs and loads.
+    constexpr int NP = kPPProducers, NC = kPPConsumers;
+    constexpr int CG = M / 4;                  // column groups of four (producers)
     constexpr int NF4 = BJ * M / 4;            // float4 per residual block
-    constexpr int PER = NF4 / NT;              // float4 per producer thread
+    constexpr int PER = NF4 / NP;              // float4 per producer thread
     constexpr int TR = 8;                      // tile rows per consumer thread
-    constexpr int NTILE = (BJ / TR) * CG;      // consumer tiles (<= NT; the rest of the consumers idle)
-    static_assert(NF4 % NT == 0 && NT % CG == 0 && NTILE <= NT, "block shape");
+    constexpr int TC = M == 64 ? 8 : 4;        // tile columns
+    constexpr int TG = M / TC;                 // tiles across
+    static_assert(NF4 % NP == 0 && NP % CG == 0 && (BJ / TR) * TG == NC, "block shape");
     static_assert(BJ % SB == 0 && SB % TR == 0, "tiles within one block-Jacobi block");
-    static_assert(!WY || NT == 2 * BJ, "the y product splits each block's columns over two halves of the consumers");
+    static_assert(!WY || NC == BJ, "the y product: one consumer per row");
     constexpr int MS = BJ * SB;                // floats of M^{-1} per stage (BJ / SB blocks of SB x SB)
     extern __shared__ __align__(128) unsigned char pp_sh[];
     float *stage0 = reinterpret_cast<float *>(pp_sh);
     float *stage1 = stage0 + MS + BJ * M;
     float *ys = stage1 + MS + BJ * M;          // 2 x BJ: the y column's residual blocks
-    float *yp = ys + 2 * BJ;                   // 2 x 2 x BJ: halves of z_y = M^{-1} r_y
-    uint64_t *bar = reinterpret_cast<uint64_t *>(yp + 4 * BJ);
+    uint64_t *bar = reinterpret_cast<uint64_t *>(ys + 2 * BJ);
     const int tid = threadIdx.x;
-    const bool producer = tid >= NT;
-    const int t = producer ? tid - NT : tid;
-    const int cg = t % CG;                     // this thread's four columns, in either role
-    double dacc[4] = {0.0, 0.0, 0.0, 0.0};     // r^T r (producers) or r^T z (consumers)
+    const bool producer = tid >= NC;
+    const int t = producer ? tid - NC : tid;
+    const int cg = t % CG;                     // a producer's four columns
+    double dacc[TC];                           // r^T r (producers: four columns) or r^T z (consumers)
+#pragma unroll
+    for (int q = 0; q < TC; ++q) dacc[q] = 0.0;
     double ydacc = 0.0;                        // the y column's r^T r (producers) or r^T z (consumers)
     const int64_t nmine = (int64_t)blockIdx.x < nblk ? (nblk - 1 - blockIdx.x) / gridDim.x + 1 : 0;
 
@@ -2412,7 +2424,7 @@ k_pc_probe(int64_t n, int64_t nblk, const float *__restrict__ Minv32, float *__r
             float4 q4[PER];
 #pragma unroll
             for (int j = 0; j < PER; ++j) {
-                const int e = t + j * NT;
+                const int e = t + j * NP;
                 q4[j] = e / CG < nb ? reinterpret_cast<const float4 *>(qz + i0 * M)[e] : make_float4(0.f, 0.f, 0.f, 0.f);
             }
             // the y column's row i0 + t (the same arithmetic as the y column's own PCG step)
@@ -2435,7 +2447,7 @@ k_pc_probe(int64_t n, int64_t nblk, const float *__restrict__ Minv32, float *__r
             float srr[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
             for (int j = 0; j < PER; ++j) {
-                const int e = t + j * NT;
+                const int e = t + j * NP;
                 float4 r4 = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (e / CG < nb) {
                     r4 = reinterpret_cast<const float4 *>(R)[e];
@@ -2471,23 +2483,21 @@ k_pc_probe(int64_t n, int64_t nblk, const float *__restrict__ Minv32, float *__r
                 for (uint32_t par = 0; par < 2; ++par) mbar_wait_bounded(&bar[b], par);
         }
     } else {
-        const int rg = t / CG;                 // rows TR rg .. TR rg + TR - 1, columns 4 cg .. 4 cg + 3
-        const int i0t = rg * TR, c0 = cg * 4;
-        const bool has_tile = t < NTILE;
+        const int i0t = (t / TG) * TR;         // rows i0t .. i0t + TR - 1
+        const int c0 = (t % TG) * 4;           // columns c0 .. c0 + 3 (and M / 2 further)
         for (int64_t k = 0; k < nmine; ++k) {
             const float *MT = (k & 1) ? stage1 : stage0;
             const float *R = MT + MS;
             const int64_t i0 = (blockIdx.x + k * gridDim.x) * BJ;
             const int nb = (int)(n - i0 < BJ ? n - i0 : BJ);
             asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)(k & 1)), "r"(kPPThreads) : "memory");
-            if (has_tile) {
             // z = M^{-1} r (symmetric M^{-1}: row kk of the stage is column kk), rows in pairs with
             // packed FP32x2 FMAs (each half rounds like fmaf)
-            float2 acc[TR / 2][4];
+            float2 acc[TR / 2][TC];
 #pragma unroll
             for (int a = 0; a < TR / 2; ++a)
 #pragma unroll
-                for (int q = 0; q < 4; ++q) acc[a][q] = make_float2(0.f, 0.f);
+                for (int q = 0; q < TC; ++q) acc[a][q] = make_float2(0.f, 0.f);
             // the tile's rows lie in block sb of the stage: M^{-1}_sb (SB x SB, symmetric) times
             // the block's SB residual rows
             const int sb = i0t / SB;
@@ -2497,88 +2507,103 @@ k_pc_probe(int64_t n, int64_t nblk, const float *__restrict__ Minv32, float *__r
             for (int kk = 0; kk < SB; ++kk) {
                 const float4 m0 = *reinterpret_cast<const float4 *>(MB + kk * SB);
                 const float4 m1 = *reinterpret_cast<const float4 *>(MB + kk * SB + 4);
-                const float4 rv = *reinterpret_cast<const float4 *>(RB + kk * M);
                 const float2 mp[4] = {make_float2(m0.x, m0.y), make_float2(m0.z, m0.w), make_float2(m1.x, m1.y),
                                       make_float2(m1.z, m1.w)};
-                const float ra[4] = {rv.x, rv.y, rv.z, rv.w};
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const float2 rq = make_float2(ra[q], ra[q]);
+                for (int h = 0; h < TC / 4; ++h) {
+                    const float4 rv = *reinterpret_cast<const float4 *>(RB + kk * M + h * (M / 2));
+                    const float ra[4] = {rv.x, rv.y, rv.z, rv.w};
 #pragma unroll
-                    for (int a = 0; a < TR / 2; ++a) acc[a][q] = __ffma2_rn(mp[a], rq, acc[a][q]);
+                    for (int q = 0; q < 4; ++q) {
+                        const float2 rq = make_float2(ra[q], ra[q]);
+#pragma unroll
+                        for (int a = 0; a < TR / 2; ++a) acc[a][4 * h + q] = __ffma2_rn(mp[a], rq, acc[a][4 * h + q]);
+                    }
                 }
             }
-            float srz[4] = {0.f, 0.f, 0.f, 0.f};
+            float srz[TC];
+#pragma unroll
+            for (int q = 0; q < TC; ++q) srz[q] = 0.f;
 #pragma unroll
             for (int a = 0; a < TR; ++a) {
                 const int i = i0t + a;
                 if (i >= nb) continue;
-                const float z[4] = {(a & 1) ? acc[a / 2][0].y : acc[a / 2][0].x, (a & 1) ? acc[a / 2][1].y : acc[a / 2][1].x,
-                                    (a & 1) ? acc[a / 2][2].y : acc[a / 2][2].x, (a & 1) ? acc[a / 2][3].y : acc[a / 2][3].x};
-                *reinterpret_cast<float4 *>(zz + (i0 + i) * M + c0) = make_float4(z[0], z[1], z[2], z[3]);
-                const float4 rv = *reinterpret_cast<const float4 *>(R + i * M + c0);
-                srz[0] = fmaf(rv.x, z[0], srz[0]);
-                srz[1] = fmaf(rv.y, z[1], srz[1]);
-                srz[2] = fmaf(rv.z, z[2], srz[2]);
-                srz[3] = fmaf(rv.w, z[3], srz[3]);
+#pragma unroll
+                for (int h = 0; h < TC / 4; ++h) {
+                    float z[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) z[q] = (a & 1) ? acc[a / 2][4 * h + q].y : acc[a / 2][4 * h + q].x;
+                    const int c = c0 + h * (M / 2);
+                    *reinterpret_cast<float4 *>(zz + (i0 + i) * M + c) = make_float4(z[0], z[1], z[2], z[3]);
+                    const float4 rv = *reinterpret_cast<const float4 *>(R + i * M + c);
+                    srz[4 * h + 0] = fmaf(rv.x, z[0], srz[4 * h + 0]);
+                    srz[4 * h + 1] = fmaf(rv.y, z[1], srz[4 * h + 1]);
+                    srz[4 * h + 2] = fmaf(rv.z, z[2], srz[4 * h + 2]);
+                    srz[4 * h + 3] = fmaf(rv.w, z[3], srz[4 * h + 3]);
+                }
             }
 #pragma unroll
-            for (int q = 0; q < 4; ++q) dacc[q] += (double)srz[q];
-            }
-            float yri = 0.0f;
+            for (int q = 0; q < TC; ++q) dacc[q] += (double)srz[q];
+            float yri = 0.0f, zyt = 0.0f;
             if (WY) {
-                // half h = t / BJ of z_y[i] = sum_kk M^{-1}_sb[kk][i] r_y[kk] over row i's block sb,
-                // kk in [h SB/2, (h+1) SB/2)
-                const int i = t % BJ, h = t / BJ;
-                const int sb = i / SB, il = i - sb * SB;
-                const float *yrs = ys + (k & 1) * BJ + sb * SB;
-                const float *MB = MT + sb * SB * SB + il;
-                float zp = 0.0f;
+                // z_y[t] = sum_kk M^{-1}_sb[kk][t] r_y[kk] over row t's block: the block's two halves apart
+                const int yb = t / SB, il = t - yb * SB;
+                const float *yrs = ys + (k & 1) * BJ + yb * SB;
+                const float *YB = MT + yb * SB * SB + il;
+                float z0 = 0.0f, z1 = 0.0f;
 #pragma unroll 8
-                for (int kk = h * (SB / 2); kk < (h + 1) * (SB / 2); ++kk) zp = fmaf(MB[kk * SB], yrs[kk], zp);
-                yp[((k & 1) * 2 + h) * BJ + i] = zp;
-                if (t < BJ) yri = ys[(k & 1) * BJ + t];
+                for (int kk = 0; kk < SB / 2; ++kk) {
+                    z0 = fmaf(YB[kk * SB], yrs[kk], z0);
+                    z1 = fmaf(YB[(kk + SB / 2) * SB], yrs[kk + SB / 2], z1);
+                }
+                zyt = z0 + z1;
+                yri = ys[(k & 1) * BJ + t];
             }
             // every consumer is done with the stage: refill it with block k + 2
-            asm volatile("bar.sync 3, %0;" ::"r"(NT) : "memory");
+            asm volatile("bar.sync 3, %0;" ::"r"(NC) : "memory");
             if (t == 0 && k + 2 < nmine) {
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 issue(k + 2);
             }
             if (WY && t < nb) {
-                const float z = yp[((k & 1) * 2) * BJ + t] + yp[((k & 1) * 2 + 1) * BJ + t];
-                zy[i0 + t] = z;
-                ydacc = fma((double)yri, (double)z, ydacc);
+                zy[i0 + t] = zyt;
+                ydacc = fma((double)yri, (double)zyt, ydacc);
             }
         }
     }
     __syncthreads();
     // per-column partials of this CTA in thread order: r^T z from the consumers, r^T r from the producers
-    double *red = reinterpret_cast<double *>(stage0);
+    double *red = reinterpret_cast<double *>(stage0);   // consumers NC x TC, producers NP x 4
+    double *redp = red + (size_t)NC * TC;
+    if (producer) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) red[(size_t)tid * 4 + q] = dacc[q];
+        for (int q = 0; q < 4; ++q) redp[(size_t)t * 4 + q] = dacc[q];
+    } else {
+#pragma unroll
+        for (int q = 0; q < TC; ++q) red[(size_t)t * TC + q] = dacc[q];
+    }
     __syncthreads();
     if (tid < M) {
-        const int g = tid / 4, q = tid % 4;
+        // column tid: run h = tid / (M / 2) of the tiles when they hold two
+        const int h = TC == 8 ? tid / (M / 2) : 0, cc = tid - h * (M / 2);
+        const int g = cc / 4, q = cc % 4;
         double s1 = 0.0, s2 = 0.0;
-        for (int u = g; u < NT; u += CG) {
-            s1 += red[(size_t)u * 4 + q];
-            s2 += red[(size_t)(NT + u) * 4 + q];
-        }
+        for (int u = g; u < NC; u += TG) s1 += red[(size_t)u * TC + 4 * h + q];
+        for (int u = tid / 4; u < NP; u += CG) s2 += redp[(size_t)u * 4 + tid % 4];
         part_rz[(int64_t)(tid + 1) * pstride + blockIdx.x] = s1;
         part_rr[(int64_t)(tid + 1) * pstride + blockIdx.x] = s2;
     }
     if (WY) {
-        // the y column's partials: consumers' r^T z, then producers' r^T r, each in thread order
+        // the y column's partials: consumers' r^T z and producers' r^T r, each by warp trees and the warps
+        // in order (one thread adding all of them took 17 us: 64 cycles an addition)
         __syncthreads();
-        red[tid] = ydacc;
+        const double yw = warp_sum(ydacc);
+        if ((tid & 31) == 0) red[tid >> 5] = yw;
         __syncthreads();
         if (tid == 0) {
             double s1 = 0.0, s2 = 0.0;
-            for (int u = 0; u < NT; ++u) {
-                s1 += red[u];
-                s2 += red[NT + u];
-            }
+            for (int w = 0; w < NC / kWarp; ++w) s1 += red[w];
+            for (int w = NC / kWarp; w < kPPThreads / kWarp; ++w) s2 += red[w];
             part_rz[blockIdx.x] = s1;
             part_rr[blockIdx.x] = s2;
         }
@@ -2878,7 +2903,7 @@ gp2s_status cg_run(gp2s_ctx *c, int m, const V *val, const CGBuffers &B, const d
     const bool pc_async = pc_avail && c->pc_async && (m == 32 || m == 64) &&
                           (bjz == 128 || (bjz == 64 && c->pc_async64));
     const int64_t nstage = ceil_div(n, (int64_t)128);   // the bulk-copy kernel's 128-row stages
-    const int pga = (int)std::min<int64_t>(c->num_sms, nstage);
+    const int pga = (int)std::min<int64_t>((int64_t)c->num_sms * (bjz == 64 && m == 32 ? pp_ctas<64, 32> : 1), nstage);
     int *dev_err = flags + 3;
     // the y column's PCG update joins the probe group's step when both use the same factors
     const bool pc_fuse_y = pcy && bjy == bjz && c->pc_fuse_y;
