@@ -59,7 +59,7 @@ typedef enum {
 typedef enum {
     GP2S_PREC_FP64 = 0,   /* FP64 values, FP64 SpMV/CG (the plain FP64 GPU form) */
     GP2S_PREC_MIXED = 1   /* FP32 values + int32 indices for assembly/SpMM/CG; FP64 dots, FP64
-                             residual refinement, FP64 tridiagonal eigensolve and reductions */
+                             residual refinement, FP64 tridiagonal quadrature and reductions */
 } gp2s_precision;
 
 typedef enum {
@@ -69,7 +69,9 @@ typedef enum {
 
 typedef enum {
     GP2S_LOGDET_AUTO = 0,   /* EXACT when n <= n_exact, else SLQ */
-    GP2S_LOGDET_EXACT = 1,  /* dense FP64 Cholesky of A: log|A| = 2 sum log L_ii */
+    GP2S_LOGDET_EXACT = 1,  /* FP64 Cholesky of A (sparse, by tiles): log|A| = 2 sum log L_ii; refused
+                               (GP2S_ENOMEM) where n^2 doubles exceed the device memory or
+                               GP2S_MEM_LIMIT */
     GP2S_LOGDET_SLQ = 2     /* stochastic Lanczos quadrature on D^{-1/2} A D^{-1/2} */
 } gp2s_logdet_method;
 
@@ -268,7 +270,7 @@ gp2s_status gp2s_solve(gp2s_ctx *ctx, const double *y, double *a, gp2s_solve_inf
 
 /*
  * log|A| of the last assembled matrix (Sec. 3; the method is left open in Sec. 4.6 / App. B.7):
- * EXACT = dense FP64 Cholesky; SLQ = stochastic Lanczos quadrature with opts->probes Rademacher
+ * EXACT = FP64 Cholesky by tiles; SLQ = stochastic Lanczos quadrature with opts->probes Rademacher
  * probes (SplitMix64, seed) and opts->lanczos_steps steps on Ah, plus sum log D_ii.
  *   logdet: host.  stderr_hat: host, optional (0 for EXACT).
  */
@@ -406,7 +408,8 @@ gp2s_status gp2s_mcmc(gp2s_ctx *ctx, int64_t n, const double *X, const double *y
  *   X_dev (n x d FP64), y_dev (n FP64): DEVICE pointers, original point order.
  *   hyper: host, as for gp2s_lml; the product kernel family only (WENDCONV returns GP2S_EINVAL).
  *   out_dev: DEVICE pointer to 3 doubles receiving {LML, y^T A^{-1} y, log|A|}; NaN if a Cholesky
- *   pivot is not positive.
+ *   pivot is not positive (or a wait inside the factorisation gave up, which overlapping calls, see
+ *   below, can bring about).
  *   cuda_stream: the stream all work is issued on (NULL = legacy default stream).  It must belong
  *   to the calling thread's current device: a stream of another device returns GP2S_EINVAL when
  *   it is not being captured.  While it is being captured this is not checked (the runtime does

@@ -27,7 +27,10 @@ namespace gp2s {
 namespace {
 
 constexpr int kCholThreads = 128;
-constexpr int kCholMaxSpins = 1 << 23;   // polls of a flag before a wait gives up (several seconds)
+// polls of a flag before a wait gives up: several seconds, and some 50 ms with every tile present (at most
+// 16 tile columns, under a millisecond; calls that overlap on the allocation-free path's one scratch array
+// clear each other's flags)
+template <bool ALL> constexpr int kCholMaxSpins = ALL ? 1 << 16 : 1 << 23;
 enum { CT_FACTOR = 0, CT_FORWARD = 1, CT_BACKWARD = 2 };
 
 __device__ __forceinline__ int ld_acquire(const int *p)
@@ -43,9 +46,10 @@ __device__ __forceinline__ void st_release(int *p, int v)
 }
 
 // Bounded wait of one thread for *flag; false when it gave up or another CTA did.
+template <bool ALL>
 __device__ __forceinline__ bool chol_wait(const int *flag, const int *abort_word)
 {
-    for (int spin = 0; spin < kCholMaxSpins; ++spin) {
+    for (int spin = 0; spin < kCholMaxSpins<ALL>; ++spin) {
         if (ld_acquire(flag)) return true;
         if ((spin & 63) == 63 && ld_acquire(abort_word)) return false;
         if (spin > 16) __nanosleep(100);
@@ -171,8 +175,8 @@ k_chol(const CholArgs a)
     // every thread learns whether thread 0's wait succeeded
     auto wait_all = [&](const int *f1, const int *f2) -> bool {
         if (tid == 0) {
-            bool ok = chol_wait(f1, abort_word);
-            if (ok && f2) ok = chol_wait(f2, abort_word);
+            bool ok = chol_wait<ALL>(f1, abort_word);
+            if (ok && f2) ok = chol_wait<ALL>(f2, abort_word);
             s_ok = ok;
         }
         __syncthreads();
