@@ -312,7 +312,7 @@ void gp2s_destroy(gp2s_ctx *c)
                       &c->val32, &c->val64, &c->counters, &c->vec, &c->vec64, &c->partials, &c->scal,
                       &c->Z, &c->Zf, &c->rec, &c->rsplit, &c->dense, &c->chol_ints, &c->H, &c->gpart,
                       &c->rb_cnt, &c->rb_ptr, &c->rb_col, &c->rb_val, &c->rb_tpart, &c->rb_seg,
-                      &c->bj_Minv, &c->bj_ld, &c->bj_Minv_y, &c->post_X, &c->post_B, &c->post_cnt,
+                      &c->bj_Minv, &c->bj_Minv_y, &c->post_X, &c->post_B, &c->post_cnt,
                       &c->post_part, &c->mr_vec, &c->mc_X, &c->mc_y, &c->wc_lam, &c->wc_sig, &c->ff_mask,
                       &c->ff_flag, &c->ff_mptr, &c->ff_mcol, &c->ff_ucnt, &c->ff_uptr, &c->ff_ucol};
     for (DevBuf *b : bufs) free_buf(*b);

@@ -116,12 +116,11 @@ struct gp2s_ctx {
     gp2s::DevBuf rb_cnt, rb_ptr, rb_col, rb_val, rb_tpart, rb_seg;
     bool rb_valid = false;
     int64_t rb_entries = 0;
-    // block-Jacobi preconditioner: FP32 M^{-1} per 64-row block and the block log-determinants
-    gp2s::DevBuf bj_Minv, bj_ld, bj_Minv_y;
+    // block-Jacobi preconditioner: FP32 M^{-1} per block
+    gp2s::DevBuf bj_Minv, bj_Minv_y;
     bool bj_valid = false;
     int bj_size = 64;               // rows per block-Jacobi block of the probe columns
     int bj_size_y = 64;             // rows per block of the y column (64 or 128)
-    double bj_logdet = 0.0;
     bool probes_for_grad = false;   // the probe solves feed the Hutchinson gradient
     bool use_graphs = true;         // replay runs of CG iterations as CUDA graphs (GP2S_GRAPHS=0: off)
     bool pc_async = true;           // probe-group PCG step on the bulk-copy pipelined kernel

@@ -1953,81 +1953,214 @@ gp2s_status launch_rb4_et(gp2s_ctx *c, const CGBuffers &B, double *part, int pst
 constexpr int kPCThreads = 256;
 
 // One CTA per block of BJ rows (BJ = 64 or 128): the dense block of Ah (FP32 values) from the
-// CSR, Cholesky L L^T, L^{-1} in place, then M^{-1} = L^{-T} L^{-1} (symmetric bit for bit: both
-// triangles come from the same products in the same order) and the block's log|M_b|.  FP32 is
-// enough for a preconditioner (a block's condition number is bounded by about 1 / sigma^2 of the
-// Jacobi-scaled matrix) and runs on the full-rate FP32 pipes; rows beyond n (last block) are
-// padded with the identity.
+// CSR, Cholesky L L^T, V = L^{-1}, then M^{-1} = V^T V (symmetric bit for bit: both triangles come
+// from the same products in the same order).  FP32 is enough for a preconditioner (a block's
+// condition number is bounded by about 1 / sigma^2 of the Jacobi-scaled matrix) and runs on the
+// full-rate FP32 pipes; rows beyond n (last block) are padded with the identity.
+//
+// What bounds it: shared-memory loads and the serial chains of a small factorisation (BJ pivots, then
+// BJ dependent sums a row), not HBM.  So each phase keeps operands in registers:
+//  - the factor goes by panels of 8 columns.  A thread owns a row of the panel and redoes the 8 x 8
+//    pivot block itself, so a panel has no barrier inside; the trailing update adds a panel's 8 terms
+//    to an element in one visit, a lane per row, the panel's rows as broadcast 16-byte loads;
+//  - V's rows are independent: a thread owns row i and walks its columns from i - 1 down with no block
+//    barrier.  V_ij is kept at S[j][i], the triangle that L leaves free, where a warp's lanes are
+//    neighbours; column j of L is copied into the warp's own buffer for 16-byte broadcasts, and the
+//    warp's own 32 x 32 corner of V stays in registers;
+//  - V^T V takes register tiles of 8 x 4, and starts each at the first k where both rows can be nonzero.
+// Every element is the same sequence of fused multiply-adds (pivots or k ascending), division and square
+// root as one element at a time would take, so M^{-1} does not depend on the blocking.
+// Measured (one element at a time, a barrier per pivot -> this): 128-row blocks, 1M points 11.8 -> 3.7 ms;
+// 64-row blocks, 8M points 25 -> 17 ms, which waits for the chains of global loads of the CSR rows.
+template <int BJ> constexpr int kBJThreads = 2 * BJ;
+constexpr int kBJPanel = 8;
+template <int BJ> constexpr size_t bj_build_smem() { return sizeof(float) * ((size_t)BJ * (BJ + 1) + BJ * kBJPanel); }
 template <int BJ>
-__global__ void __launch_bounds__(kPCThreads)
+__global__ void __launch_bounds__(kBJThreads<BJ>, BJ == 128 ? 3 : 6)
 k_bj_build(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col, const float *__restrict__ val32,
-           int64_t n, float *__restrict__ Minv32, double *__restrict__ logdet_blk,
-           int *__restrict__ bad)
+           int64_t n, float *__restrict__ Minv32, int *__restrict__ bad)
 {
-    extern __shared__ float bjf_sh[];
-    float (*S)[BJ + 1] = reinterpret_cast<float (*)[BJ + 1]>(bjf_sh);   // L, then L^{-1} (lower)
-    float *tmp = bjf_sh + BJ * (BJ + 1);                                // one column of L
+    constexpr int NT = kBJThreads<BJ>, NW = NT / kWarp, PW = kBJPanel;
+    extern __shared__ __align__(16) float bjf_sh[];
+    float (*S)[BJ + 1] = reinterpret_cast<float (*)[BJ + 1]>(bjf_sh);   // L below, V^T above the diagonal
+    float *P = bjf_sh + BJ * (BJ + 1);                                  // a panel's rows; then columns of L
     const int64_t b = blockIdx.x;
     const int64_t i0 = b * BJ;
     const int nb = (int)(n - i0 < BJ ? n - i0 : BJ);
-    for (int t = threadIdx.x; t < BJ * BJ; t += blockDim.x) {
-        int i = t / BJ, j = t % BJ;
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    for (int e = t; e < BJ * BJ; e += NT) {
+        const int i = e / BJ, j = e % BJ;
         S[i][j] = (i == j && i >= nb) ? 1.0f : 0.0f;
     }
     __syncthreads();
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int i = wid; i < nb; i += kPCThreads / kWarp) {
+    for (int i = wid; i < nb; i += NW) {
         for (int p = rowptr[i0 + i] + lane; p < rowptr[i0 + i + 1]; p += kWarp) {
-            int64_t j = col[p] - i0;
-            if (j >= 0 && j < nb) S[i][j] = val32[p];
+            const int64_t j = col[p] - i0;
+            if (j >= 0 && j <= i) S[i][j] = val32[p];
         }
     }
     __syncthreads();
-    // right-looking Cholesky of the lower triangle; the trailing update visits only the
-    // (BJ - j - 1)^2 square below and right of the pivot
-    for (int j = 0; j < BJ; ++j) {
-        if (threadIdx.x == 0) {
-            float d = S[j][j];
-            if (!(d > 0.0f)) { atomicOr(bad, 1); d = 1.0f; }
-            S[j][j] = sqrtf(d);
+    for (int p0 = 0; p0 < BJ; p0 += PW) {
+        float x[PW];
+        if (t < BJ && (t | 31) >= p0) {
+            float D[PW][PW];
+#pragma unroll
+            for (int a = 0; a < PW; ++a) {
+                x[a] = S[t][p0 + a];
+#pragma unroll
+                for (int k = 0; k <= a; ++k) D[a][k] = S[p0 + a][p0 + k];
+            }
+#pragma unroll
+            for (int j = 0; j < PW; ++j) {
+                float d = D[j][j];
+                if (!(d > 0.0f)) {
+                    if (t == p0) atomicOr(bad, 1);
+                    d = 1.0f;
+                }
+                d = sqrtf(d);
+#pragma unroll
+                for (int a = j + 1; a < PW; ++a) D[a][j] /= d;
+                x[j] = t == p0 + j ? d : x[j] / d;
+#pragma unroll
+                for (int a = j + 1; a < PW; ++a) {
+#pragma unroll
+                    for (int k = j + 1; k <= a; ++k) D[a][k] = fmaf(-D[a][j], D[k][j], D[a][k]);
+                    x[a] = fmaf(-x[j], D[a][j], x[a]);
+                }
+            }
+            if (t >= p0 + PW) {
+#pragma unroll
+                for (int a = 0; a < PW; ++a) S[t][p0 + a] = x[a];
+#pragma unroll
+                for (int a = 0; a < PW; a += 4)
+                    *reinterpret_cast<float4 *>(P + t * PW + a) = make_float4(x[a], x[a + 1], x[a + 2], x[a + 3]);
+            }
         }
         __syncthreads();
-        for (int i = j + 1 + threadIdx.x; i < BJ; i += blockDim.x) S[i][j] /= S[j][j];
-        __syncthreads();
-        const int w = BJ - j - 1;
-        for (int t = threadIdx.x; t < w * w; t += blockDim.x) {
-            const int i = j + 1 + t / w, k = j + 1 + t % w;
-            if (k <= i) S[i][k] -= S[i][j] * S[k][j];
+        // the pivot block's own rows, once every thread has read them
+        if (t >= p0 && t < p0 + PW) {
+#pragma unroll
+            for (int a = 0; a < PW; ++a)
+                if (p0 + a <= t) S[t][p0 + a] = x[a];
+        }
+        // trailing update, 32 rows x 8 columns a warp (elements above the diagonal hold nothing yet)
+        int u = wid;
+        for (int g = (p0 + PW) / 32; g < BJ / 32; ++g) {
+            const int nc = (32 * g + 32 - p0 - PW) / 8;
+            const int i = 32 * g + lane;
+            if (u < nc) {
+                float l[PW];
+#pragma unroll
+                for (int a = 0; a < PW; ++a) l[a] = S[i][p0 + a];
+                for (; u < nc; u += NW) {
+                    const int c0 = p0 + PW + 8 * u;
+#pragma unroll
+                    for (int k = c0; k < c0 + 8; ++k) {
+                        const float4 pa = *reinterpret_cast<const float4 *>(P + k * PW);
+                        const float4 pb = *reinterpret_cast<const float4 *>(P + k * PW + 4);
+                        float v = S[i][k];
+                        v = fmaf(-l[0], pa.x, v);
+                        v = fmaf(-l[1], pa.y, v);
+                        v = fmaf(-l[2], pa.z, v);
+                        v = fmaf(-l[3], pa.w, v);
+                        v = fmaf(-l[4], pb.x, v);
+                        v = fmaf(-l[5], pb.y, v);
+                        v = fmaf(-l[6], pb.z, v);
+                        v = fmaf(-l[7], pb.w, v);
+                        S[i][k] = v;
+                    }
+                }
+            }
+            u -= nc;
         }
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        double ld = 0.0;
-        for (int i = 0; i < nb; ++i) ld += log((double)S[i][i]);
-        logdet_blk[b] = 2.0 * ld;
-    }
-    // V = L^{-1} in place, columns from the last to the first: V L = I gives V_jj = 1 / L_jj and
-    // V_ij = -(sum_{k=j+1..i} V_ik L_kj) / L_jj, which needs only the columns of V to the right of
-    // j (already in place) and column j of L (saved in tmp first).
-    for (int j = BJ - 1; j >= 0; --j) {
-        for (int k = j + threadIdx.x; k < BJ; k += blockDim.x) tmp[k] = S[k][j];
-        __syncthreads();
-        const float ljj = tmp[j];
-        for (int i = j + 1 + threadIdx.x; i < BJ; i += blockDim.x) {
+    // V = L^{-1} from V L = I: V_ii = 1 / L_ii and, for j from i - 1 down,
+    // V_ij = -(sum_{k=j+1..i} V_ik L_kj) / L_jj
+    float vii = 1.0f;
+    if (t < BJ) {
+        const int i = t, w32 = t & ~31;
+        float *cb = P + wid * BJ;                       // column j of L
+        vii = 1.0f / S[i][i];
+        for (int j = w32 + 30; j >= w32; --j) {         // columns of the warp's own corner
+            __syncwarp();
+            if (w32 + lane >= j) cb[w32 + lane] = S[w32 + lane][j];
+            __syncwarp();
             float s = 0.0f;
-            for (int k = j + 1; k <= i; ++k) s = fmaf(S[i][k], tmp[k], s);
-            S[i][j] = -s / ljj;
+            for (int k = j + 1; k < w32 + 32; ++k)
+                if (k <= i) s = fmaf(k < i ? S[k][i] : vii, cb[k], s);
+            if (i > j) S[j][i] = -s / cb[j];
         }
-        if (threadIdx.x == 0) S[j][j] = 1.0f / ljj;
-        __syncthreads();
+        float vd[32];
+#pragma unroll
+        for (int k = 0; k < 32; ++k) vd[k] = k < lane ? S[w32 + k][i] : k == lane ? vii : 0.0f;
+        for (int j = w32 - 1; j >= 0; --j) {
+            __syncwarp();
+            for (int k = (j & ~31) + lane; k < w32 + 32; k += 32)
+                if (k >= j) cb[k] = S[k][j];
+            __syncwarp();
+            float s = 0.0f;
+            int k = j + 1;
+            for (; k & 3; ++k) s = fmaf(S[k][i], cb[k], s);   // w32 is a multiple of 4
+#pragma unroll 4
+            for (; k < w32; k += 4) {
+                const float4 l4 = *reinterpret_cast<const float4 *>(cb + k);
+                s = fmaf(S[k][i], l4.x, s);
+                s = fmaf(S[k + 1][i], l4.y, s);
+                s = fmaf(S[k + 2][i], l4.z, s);
+                s = fmaf(S[k + 3][i], l4.w, s);
+            }
+#pragma unroll
+            for (int q = 0; q < 32; q += 4) {
+                const float4 l4 = *reinterpret_cast<const float4 *>(cb + w32 + q);
+                s = fmaf(vd[q], l4.x, s);
+                s = fmaf(vd[q + 1], l4.y, s);
+                s = fmaf(vd[q + 2], l4.z, s);
+                s = fmaf(vd[q + 3], l4.w, s);
+            }
+            S[j][i] = -s / cb[j];
+        }
     }
+    __syncthreads();
+    for (int e = t; e < BJ * BJ; e += NT) {
+        const int i = e / BJ, j = e % BJ;
+        if (j < i) S[i][j] = 0.0f;
+    }
+    if (t < BJ) S[t][t] = vii;
+    __syncthreads();
+    // (V^T V)_ij = sum_k S[i][k] S[j][k], k >= max(i, j)
+    constexpr int TY = NT / 16, NA = BJ / TY, NB = 4;   // thread rows ty + TY a, columns tx + 16 b
+    const int tx = t & 15, ty = t >> 4;
     float *Mb = Minv32 + b * BJ * BJ;
-    for (int t = threadIdx.x; t < BJ * BJ; t += blockDim.x) {
-        int i = t / BJ, j = t % BJ;
-        // (L^{-T} L^{-1})_ij = sum_k V[k][i] V[k][j], k >= max(i, j)
-        float s = 0.0f;
-        for (int k = i > j ? i : j; k < BJ; ++k) s = fmaf(S[k][i], S[k][j], s);
-        Mb[t] = s;
+#pragma unroll
+    for (int h = 0; h < BJ / (16 * NB); ++h) {
+        float acc[NA][NB];
+#pragma unroll
+        for (int a = 0; a < NA; ++a)
+#pragma unroll
+            for (int q = 0; q < NB; ++q) acc[a][q] = 0.0f;
+#pragma unroll
+        for (int kb = h * NB; kb < BJ / 16; ++kb) {
+#pragma unroll 2
+            for (int k = 16 * kb; k < 16 * kb + 16; ++k) {
+                float rv[NA], cv[NB];
+#pragma unroll
+                for (int a = 0; a < NA; ++a)
+                    if (TY * a < 16 * kb + 16) rv[a] = S[ty + TY * a][k];
+#pragma unroll
+                for (int q = 0; q < NB; ++q)
+                    if (h * NB + q <= kb) cv[q] = S[tx + 16 * (h * NB + q)][k];
+#pragma unroll
+                for (int a = 0; a < NA; ++a)
+#pragma unroll
+                    for (int q = 0; q < NB; ++q)
+                        if (TY * a < 16 * kb + 16 && h * NB + q <= kb) acc[a][q] = fmaf(rv[a], cv[q], acc[a][q]);
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < NA; ++a)
+#pragma unroll
+            for (int q = 0; q < NB; ++q) Mb[(ty + TY * a) * BJ + tx + 16 * (h * NB + q)] = acc[a][q];
     }
 }
 
@@ -2636,38 +2769,30 @@ int bj_block_size(const gp2s_ctx *c)
 }
 
 // Build one set of block-Jacobi factors (FP32 M^{-1}) with blocks of bj rows.
-static gp2s_status build_bj_set(gp2s_ctx *c, int bj, DevBuf &minv, double *logdet)
+template <int BJ> static gp2s_status bj_build_launch(gp2s_ctx *c, int64_t nblk, DevBuf &minv, int *bad)
+{
+    constexpr size_t smem = bj_build_smem<BJ>();
+    GP2S_TRY(smem_attr(c, (const void *)k_bj_build<BJ>, smem));
+    k_bj_build<BJ><<<(unsigned)nblk, kBJThreads<BJ>, smem, c->stream>>>(c->rowptr.as<int32_t>(), c->col.as<int32_t>(),
+                                                                        c->val32.as<float>(), c->A.n, minv.as<float>(), bad);
+    GP2S_LAUNCH(c);
+    return GP2S_OK;
+}
+
+static gp2s_status build_bj_set(gp2s_ctx *c, int bj, DevBuf &minv)
 {
     const int64_t n = c->A.n;
     const int64_t nblk = ceil_div(n, bj);
     GP2S_TRY(ensure(c, minv, sizeof(float) * (size_t)nblk * bj * bj));
-    GP2S_TRY(ensure(c, c->bj_ld, sizeof(double) * (size_t)nblk + 64));
     GP2S_TRY(ensure(c, c->counters, 256));
     int *bad = reinterpret_cast<int *>(c->counters.as<char>() + 208);
     GP2S_CUDA(c, cudaMemsetAsync(bad, 0, sizeof(int), c->stream));
-    const size_t smem = sizeof(float) * ((size_t)bj * (bj + 1) + bj);
-    if (bj == 128) {
-        GP2S_TRY(smem_attr(c, (const void *)k_bj_build<128>, smem));
-        k_bj_build<128><<<(unsigned)nblk, kPCThreads, smem, c->stream>>>(
-            c->rowptr.as<int32_t>(), c->col.as<int32_t>(), c->val32.as<float>(), n, minv.as<float>(),
-            c->bj_ld.as<double>(), bad);
-    } else {
-        GP2S_TRY(smem_attr(c, (const void *)k_bj_build<64>, smem));
-        k_bj_build<64><<<(unsigned)nblk, kPCThreads, smem, c->stream>>>(
-            c->rowptr.as<int32_t>(), c->col.as<int32_t>(), c->val32.as<float>(), n, minv.as<float>(),
-            c->bj_ld.as<double>(), bad);
-    }
-    GP2S_LAUNCH(c);
-    // log|M| = sum of the block log-determinants (fixed-order host sum)
-    std::vector<double> ld((size_t)nblk);
+    if (bj == 128) GP2S_TRY(bj_build_launch<128>(c, nblk, minv, bad));
+    else GP2S_TRY(bj_build_launch<64>(c, nblk, minv, bad));
     int hbad = 0;
-    GP2S_CUDA(c, cudaMemcpyAsync(ld.data(), c->bj_ld.p, sizeof(double) * nblk, cudaMemcpyDeviceToHost, c->stream));
     GP2S_CUDA(c, cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     GP2S_CUDA(c, cudaStreamSynchronize(c->stream));
     if (hbad) return set_err(c, GP2S_ENOTPD, "block-Jacobi: a diagonal block is not positive definite");
-    double s = 0.0;
-    for (double v : ld) s += v;
-    *logdet = s;
     return GP2S_OK;
 }
 
@@ -2676,11 +2801,8 @@ static gp2s_status build_bj_set(gp2s_ctx *c, int bj, DevBuf &minv, double *logde
 gp2s_status build_block_jacobi(gp2s_ctx *c)
 {
     const int bjz = bj_block_size(c), bjy = bjz;
-    GP2S_TRY(build_bj_set(c, bjz, c->bj_Minv, &c->bj_logdet));
-    if (bjy != bjz) {
-        double ldy = 0.0;
-        GP2S_TRY(build_bj_set(c, bjy, c->bj_Minv_y, &ldy));
-    }
+    GP2S_TRY(build_bj_set(c, bjz, c->bj_Minv));
+    if (bjy != bjz) GP2S_TRY(build_bj_set(c, bjy, c->bj_Minv_y));
     c->bj_size = bjz;
     c->bj_size_y = bjy;
     c->bj_valid = true;

@@ -457,6 +457,26 @@ def test_band_matrix_y_solve(gp, ctx, n, row):
     assert ctx.logdet()[0] == pytest.approx(info["logdet"], rel=1e-9, abs=1e-9)
 
 
+@pytest.mark.parametrize("bj", [64, 128])
+@pytest.mark.parametrize("n", [1, 2, 8, 9, 31, 33, 63, 64, 65, 100, 127, 128, 129, 200, 1031])
+def test_block_jacobi_factors_at_block_edges(gp, ctx, bj, n):
+    """A matrix of one block (partly filled panels, rows past n): M is A, so a step leaves the error of
+    M^{-1} in FP32, at most n eps kappa = 128 * 6e-8 * 1000 < 1e-2, and four steps reach the first tolerance
+    (1e-6) and each restart's.  More blocks, the last one ragged: the FP64 residual, formed here from the
+    CSR."""
+    w = W.random_small(830 + n, n, 2, L=3, sigma2=0.1, r=0.6 if n < 8 else None)
+    h = gp.Hyper(**w["hyper"])
+    ctx.assemble(w["X"], h, gp.default_opts(precond=2, bj_block=bj))
+    key, A64, _, _, _ = _csr_orig(ctx.csr())
+    A = np.zeros(n * n)
+    A[key] = A64
+    a, info = ctx.solve(w["y"])
+    assert info["relres"] <= 1e-8
+    assert np.linalg.norm(w["y"] - A.reshape(n, n) @ a) <= 2e-8 * np.linalg.norm(w["y"])
+    if n <= bj:
+        assert info["iters"] <= 4 * (info["outer"] + 1)
+
+
 def test_autograd_function(gp, ctx):
     w = W.random_small(303, 3000, 2, L=2, sigma2=1e-3)
     h = gp.Hyper(**w["hyper"])
