@@ -253,7 +253,7 @@ gp2s_status slq_logdet(gp2s_ctx *c, int m, int ksteps, double *logdet_hat, doubl
     GP2S_CUDA(c, cudaMemcpyAsync(g.data(), out, sizeof(double) * m, cudaMemcpyDeviceToHost, c->stream));
     GP2S_CUDA(c, cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     GP2S_CUDA(c, cudaStreamSynchronize(c->stream));
-    if (hbad) return set_err(c, GP2S_EBREAKDOWN, "SLQ: tridiagonal eigensolve failed or non-positive Ritz value");
+    if (hbad) return set_err(c, GP2S_EBREAKDOWN, "SLQ: a tridiagonal is not positive definite or not finite");
     const double n = (double)c->A.n;
     double mean = 0.0;
     for (int s = 0; s < m; ++s) mean += n * g[s];
