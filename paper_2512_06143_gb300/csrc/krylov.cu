@@ -1967,11 +1967,14 @@ constexpr int kPCThreads = 256;
 //    barrier.  V_ij is kept at S[j][i], the triangle that L leaves free, where a warp's lanes are
 //    neighbours; column j of L is copied into the warp's own buffer for 16-byte broadcasts, and the
 //    warp's own 32 x 32 corner of V stays in registers;
+//  - the CSR rows of a block are one range, read four independent entries a thread, the row found by
+//    bisection only for the entries that fall into the block;
 //  - V^T V takes register tiles of 8 x 4, and starts each at the first k where both rows can be nonzero.
 // Every element is the same sequence of fused multiply-adds (pivots or k ascending), division and square
 // root as one element at a time would take, so M^{-1} does not depend on the blocking.
-// Measured (one element at a time, a barrier per pivot -> this): 128-row blocks, 1M points 11.8 -> 3.7 ms;
-// 64-row blocks, 8M points 25 -> 17 ms, which waits for the chains of global loads of the CSR rows.
+// Measured (one element at a time, a barrier per pivot -> this): 128-row blocks, 1M points 11.8 -> 3.1 ms;
+// 64-row blocks, 8M points 25 -> 12.8 ms (3.7 and 17 with the CSR read row by row and V's corner in
+// shared memory).
 template <int BJ> constexpr int kBJThreads = 2 * BJ;
 constexpr int kBJPanel = 8;
 template <int BJ> constexpr size_t bj_build_smem() { return sizeof(float) * ((size_t)BJ * (BJ + 1) + BJ * kBJPanel); }
@@ -1992,11 +1995,30 @@ k_bj_build(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col, 
         const int i = e / BJ, j = e % BJ;
         S[i][j] = (i == j && i >= nb) ? 1.0f : 0.0f;
     }
+    int *rp = reinterpret_cast<int *>(P);               // the block's row pointers, until the first panel
+    for (int e = t; e <= nb; e += NT) rp[e] = rowptr[i0 + e];
     __syncthreads();
-    for (int i = wid; i < nb; i += NW) {
-        for (int p = rowptr[i0 + i] + lane; p < rowptr[i0 + i + 1]; p += kWarp) {
-            const int64_t j = col[p] - i0;
-            if (j >= 0 && j <= i) S[i][j] = val32[p];
+    for (int64_t e0 = rp[0] + t; e0 < rp[nb]; e0 += 4 * NT) {
+        int cj[4];
+        float cv[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int64_t p = e0 + q * NT;
+            const bool in = p < rp[nb];
+            cj[q] = in ? col[p] : -1;
+            cv[q] = in ? val32[p] : 0.0f;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int64_t j = cj[q] - i0;
+            if (j < 0 || j >= nb) continue;
+            int lo = 0, hi = nb;                        // the entry's row: the last that starts at or before it
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) / 2;
+                if (rp[mid] <= e0 + q * NT) lo = mid;
+                else hi = mid;
+            }
+            if (j <= lo) S[lo][j] = cv[q];
         }
     }
     __syncthreads();
@@ -2082,28 +2104,41 @@ k_bj_build(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ col, 
         const int i = t, w32 = t & ~31;
         float *cb = P + wid * BJ;                       // column j of L
         vii = 1.0f / S[i][i];
-        for (int j = w32 + 30; j >= w32; --j) {         // columns of the warp's own corner
-            __syncwarp();
-            if (w32 + lane >= j) cb[w32 + lane] = S[w32 + lane][j];
-            __syncwarp();
-            float s = 0.0f;
-            for (int k = j + 1; k < w32 + 32; ++k)
-                if (k <= i) s = fmaf(k < i ? S[k][i] : vii, cb[k], s);
-            if (i > j) S[j][i] = -s / cb[j];
-        }
-        float vd[32];
+        float vd[32];                                   // V_i,w32.. of the warp's own corner
 #pragma unroll
-        for (int k = 0; k < 32; ++k) vd[k] = k < lane ? S[w32 + k][i] : k == lane ? vii : 0.0f;
+        for (int j = 31; j >= 0; --j) {
+            float s = 0.0f;
+#pragma unroll
+            for (int k = j + 1; k < 32; ++k) s = fmaf(vd[k], S[w32 + k][w32 + j], s);
+            vd[j] = j < lane ? -s / S[w32 + j][w32 + j] : j == lane ? vii : 0.0f;
+        }
+#pragma unroll
+        for (int j = 0; j < 32; ++j)
+            if (j < lane) S[w32 + j][i] = vd[j];
+        float nx[BJ / 32];                              // column j of L on its way to cb
+#pragma unroll
+        for (int q = 0; q < BJ / 32; ++q)
+            nx[q] = w32 > 0 && 32 * q <= w32 && 32 * q + lane >= w32 - 1 ? S[32 * q + lane][w32 - 1] : 0.0f;
         for (int j = w32 - 1; j >= 0; --j) {
             __syncwarp();
-            for (int k = (j & ~31) + lane; k < w32 + 32; k += 32)
-                if (k >= j) cb[k] = S[k][j];
+#pragma unroll
+            for (int q = 0; q < BJ / 32; ++q)
+                if (32 * q <= w32) cb[32 * q + lane] = nx[q];
             __syncwarp();
+#pragma unroll
+            for (int q = 0; q < BJ / 32; ++q)
+                nx[q] = j > 0 && 32 * q <= w32 && 32 * q + lane >= j - 1 ? S[32 * q + lane][j - 1] : 0.0f;
             float s = 0.0f;
-            int k = j + 1;
-            for (; k & 3; ++k) s = fmaf(S[k][i], cb[k], s);   // w32 is a multiple of 4
+            const int k0 = (j + 1) & ~3;                // terms k <= j of the first four are zero
+            if (k0 < w32) {
+                const float4 l4 = *reinterpret_cast<const float4 *>(cb + k0);
+                s = fmaf(k0 > j ? S[k0][i] : 0.0f, l4.x, s);
+                s = fmaf(k0 + 1 > j ? S[k0 + 1][i] : 0.0f, l4.y, s);
+                s = fmaf(k0 + 2 > j ? S[k0 + 2][i] : 0.0f, l4.z, s);
+                s = fmaf(S[k0 + 3][i], l4.w, s);
+            }
 #pragma unroll 4
-            for (; k < w32; k += 4) {
+            for (int k = k0 + 4; k < w32; k += 4) {
                 const float4 l4 = *reinterpret_cast<const float4 *>(cb + k);
                 s = fmaf(S[k][i], l4.x, s);
                 s = fmaf(S[k + 1][i], l4.y, s);
