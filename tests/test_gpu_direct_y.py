@@ -1,0 +1,47 @@
+"""The y solve of one-dimensional points by the tiled Cholesky factor (SLQ evaluations without a gradient):
+what choosing it costs, and what happens where it cannot or should not run."""
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2512_06143_gb300 import workloads as W  # noqa: E402
+
+
+@pytest.fixture(scope="module")
+def gp():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2512_06143_gb300 as gp
+    from paper_2512_06143_gb300 import build
+    build.build()
+    gp.load()
+    return gp
+
+
+def _line(n, row, sigma2):
+    """n points in one dimension on the GPU with about `row` stored entries per row."""
+    w = W.random_small(910 + n, n, 1, L=3, sigma2=sigma2)
+    w["hyper"]["r"] *= row / 30.0
+    return torch.tensor(w["X"], device="cuda"), torch.tensor(w["y"], device="cuda"), w["hyper"]
+
+
+def test_a_new_pattern_is_ordered_in_little_time(gp):
+    """A step that moves r has a new pattern, whose elimination order is found on the host while the GPU
+    waits.  On a band of 5,625 tile rows that is a few ms of an evaluation of about 14; going through all tiles
+    at every step made the evaluation five times as long as one on the same pattern."""
+    X, y, hyper = _line(180_000, 40, 1e-3)
+    ctx = gp.Context(0)
+    opts = gp.default_opts(logdet=gp.LOGDET_SLQ, probes=16, lanczos_steps=100, seed=3)
+    r = hyper["r"]
+
+    def solve_ms(step):
+        h = gp.Hyper(**dict(hyper, r=r * (1.0 + 1e-4 * step)))
+        info = ctx.lml(X, y, h, opts)[1]
+        assert info["iters_y"] == 0 and info["relres"] <= 1e-10
+        return info["ms_solve"]
+
+    solve_ms(0)
+    new = min(solve_ms(step) for step in range(1, 5))
+    same = min(solve_ms(4) for _ in range(4))
+    assert new < 2.0 * same
