@@ -626,18 +626,28 @@ cudaError_t chol_launch(const CholArgs &a, int num_sms, cudaStream_t stream)
     return cudaGetLastError();
 }
 
+// The factorisation takes matrices whose dense form would fit in the device's memory (or in GP2S_MEM_LIMIT): the
+// order of a larger tile graph would take the host minutes.
+gp2s_status exact_fits(gp2s_ctx *c, bool *fits)
+{
+    if (!c->total_mem) {
+        size_t free_b = 0;
+        GP2S_CUDA(c, cudaMemGetInfo(&free_b, &c->total_mem));
+    }
+    const double n = (double)c->A.n;
+    *fits = 8.0 * n * n <= (double)(c->mem_limit ? c->mem_limit : c->total_mem);
+    return GP2S_OK;
+}
+
 // The plan of the current pattern in c->chol_ints, built when the pattern is new: the tile adjacency comes
 // from the GPU, the order and the task list go back.
 static gp2s_status chol_plan(gp2s_ctx *c)
 {
     if (c->chol_plan_valid) return GP2S_OK;
     const int64_t n = c->A.n;
-    // meant for matrices whose dense form would fit: the order of a larger tile graph would take the host
-    // minutes, and its factor is refused as the dense one is
-    size_t free_b = 0, total_b = 0;
-    GP2S_CUDA(c, cudaMemGetInfo(&free_b, &total_b));
-    if (8.0 * (double)n * (double)n > (double)(c->mem_limit ? c->mem_limit : total_b))
-        return set_err(c, GP2S_ENOMEM, "exact log-determinant: n^2 doubles exceed the device memory");
+    bool fits = false;
+    GP2S_TRY(exact_fits(c, &fits));
+    if (!fits) return set_err(c, GP2S_ENOMEM, "exact log-determinant: n^2 doubles exceed the device memory");
     // an entry `band` below the diagonal lies at most ceil(band / kCT) tiles below it
     const int nt = (int)ceil_div(n, kCT), words = std::max(1, (int)ceil_div(ceil_div(c->A.band, kCT), 32));
     const size_t nbits = (size_t)nt * words;

@@ -95,6 +95,7 @@ struct gp2s_ctx {
     cudaStream_t stream = nullptr;
     std::string err;
     size_t mem_limit = 0;     // GP2S_MEM_LIMIT (0 = none)
+    size_t total_mem = 0;     // the device's memory, once asked for (exact_fits)
     size_t mem_in_use = 0;
     // geometry / sort
     gp2s::DevBuf Xin, yin, keys, keys2, idx, idx2, perm, iperm;
@@ -264,6 +265,8 @@ gp2s_status minres_solve(gp2s_ctx *c, const double *b, double *x, double tol, in
 // columns to relative residual tol (xz: solutions, rz: final recursively updated residuals).
 gp2s_status krylov_columns_buffers(gp2s_ctx *c, int m, void **rz, void **xz);
 gp2s_status krylov_columns_solve(gp2s_ctx *c, int m, double tol, int *iters);
+// Whether exact_logdet_solve takes a matrix of the current size (its own buffers may still not fit).
+gp2s_status exact_fits(gp2s_ctx *c, bool *fits);
 // log|Ah| by tiled Cholesky and, with y_sorted_dev, a = A^{-1} y in vec64 slot 3 (cholesky.cu).
 gp2s_status exact_logdet_solve(gp2s_ctx *c, const double *y_sorted_dev, double *logdet_hat);
 // Reductions used by several stages

@@ -3480,7 +3480,9 @@ gp2s_status krylov_solve(gp2s_ctx *c, const double *y_sorted_dev, bool with_prob
     // an evaluation without a gradient (training, batches) on a band matrix: the probe columns run their
     // Lanczos steps beside an idle y column, and y is solved by the tiled Cholesky factor; where that fails
     // the y column's PCG follows on its own
-    const bool direct = mixed && mm > 0 && !y_zero && !c->probes_for_grad && o.precond == 2 && y_direct(c);
+    bool direct = mixed && mm > 0 && !y_zero && !c->probes_for_grad && o.precond == 2 && y_direct(c);
+    // a matrix that the factorisation refuses is PCG's from the start, beside the probes
+    if (direct) GP2S_TRY(exact_fits(c, &direct));
     if (direct) {
         GP2S_CUDA(c, cudaMemsetAsync(r64, 0, sizeof(double) * n, c->stream));
         GP2S_TRY((cg_run<float, float>(c, mm, c->val32.as<float>(), B, r64, 1.0, tol_z, ksteps, ksteps, rec, o.max_iter,

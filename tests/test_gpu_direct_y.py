@@ -45,3 +45,22 @@ def test_a_new_pattern_is_ordered_in_little_time(gp):
     new = min(solve_ms(step) for step in range(1, 5))
     same = min(solve_ms(4) for _ in range(4))
     assert new < 2.0 * same
+
+
+def test_a_matrix_that_the_factorisation_refuses_keeps_y_beside_the_probes(gp, monkeypatch):
+    """Past the size that the exact factorisation takes (8 n^2 bytes against GP2S_MEM_LIMIT) the y column shares
+    the probes' steps from the first one.  An evaluation with the gradient, which never factors, does the same
+    solves when its probes need not converge: the same steps, bit for bit (y's steps on their own go through
+    another matrix kernel, whose sums run in another order)."""
+    X, y, hyper = _line(20_000, 40, 1e-3)
+    h = gp.Hyper(**hyper)
+    opts = gp.default_opts(logdet=gp.LOGDET_SLQ, probes=16, lanczos_steps=100, seed=3, tol_probe=1.0)
+    free = gp.Context(0).lml(X, y, h, opts)[1]
+    monkeypatch.setenv("GP2S_MEM_LIMIT", str(1 << 30))
+    ctx = gp.Context(0)
+    info = ctx.lml(X, y, h, opts)[1]
+    with_grad = ctx.lml_grad(X, y, h, opts)[2]
+    assert info["iters_y"] == with_grad["iters_y"] > 0 and info["relres"] == with_grad["relres"] <= 1e-8
+    assert info["quad"] == with_grad["quad"]
+    assert info["iters_probes"] == free["iters_probes"] and info["logdet"] == pytest.approx(free["logdet"], rel=1e-12)
+    assert info["quad"] == pytest.approx(free["quad"], rel=1e-7)
