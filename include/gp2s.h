@@ -152,8 +152,8 @@ typedef struct {
     int32_t solver;          /* solver of the y column: GP2S_SOLVER_CG (default; multi-RHS with the
                                 probes, FP32 in MIXED precision with FP64 reliable updates and
                                 refinement; gp2s_lml with SLQ in MIXED precision and precond = 2 solves
-                                a band matrix, one-dimensional points, by FP64 Cholesky instead and
-                                reports no y iterations) or
+                                a band matrix, one-dimensional points, by FP64 Cholesky instead
+                                unless few iterations will do, and reports no y iterations then) or
                                 GP2S_SOLVER_MINRES (App. B.6's solver: FP64 MINRES on
                                 D^{-1/2} A D^{-1/2}, restarted on the FP64 residual until
                                 tol_refine); the probe columns always run CG */

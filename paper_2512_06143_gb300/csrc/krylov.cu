@@ -410,7 +410,7 @@ __device__ __forceinline__ void scal_alpha(int c, double s, double *__restrict__
         active[c] = 0;
         q[S_ALPHA] = 0.0;
         q[S_STOP] = 2.0;
-        if (!(q[S_RR] <= lucky * q[S_B2])) atomicOr(&flags[0], 1);   // breakdown
+        if (!(q[S_RR] <= lucky * q[S_B2])) atomicOr(&flags[0], c == 0 ? 2 : 1);   // breakdown
         return;
     }
     double a = q[S_RHO] / s;
@@ -2966,6 +2966,16 @@ struct ReliableY {
     int replacements = 0;
 };
 
+// The y column on trial: its iterations go on only while they promise to cost less than the other way to the
+// solution, which the caller then takes.  At each check the cost is that of the iterations so far, of those
+// still needed at the mean rate so far, and of `more` after them; so a column that stalls is given up
+// once it has spent `budget_us`, whatever it promised.
+struct TrialY {
+    double budget_us, it_us;  // the other way; one iteration
+    int more;                 // iterations of the refinement that follows
+    bool done = false;        // the column has converged
+};
+
 // One CG run (x0 = 0) on columns [y | probes]; the probe right-hand sides must already be in rz.
 // y_idle: rhs_y is zero, so the y column is inactive from the start and its part of every step is left out
 // (a log-determinant of 200,003 points in 2-D 26.3 -> 23.5 ms, a posterior variance of 200 points on 100,000
@@ -2973,7 +2983,7 @@ struct ReliableY {
 template <class T, class V>
 gp2s_status cg_run(gp2s_ctx *c, int m, const V *val, const CGBuffers &B, const double *rhs_y, double tol_y,
                    double tol_z, int kmin_probe, int ksteps, double *rec, int max_iter, int *iters_y,
-                   int *iters_z, bool *breakdown, ReliableY *ru = nullptr, bool y_idle = false)
+                   int *iters_z, bool *breakdown, ReliableY *ru = nullptr, bool y_idle = false, TrialY *trial = nullptr)
 {
     const Assembled &A = c->A;
     const int64_t n = A.n;
@@ -2996,7 +3006,7 @@ gp2s_status cg_run(gp2s_ctx *c, int m, const V *val, const CGBuffers &B, const d
     double *part = c->partials.as<double>();
     double *sc = c->scal.as<double>();
     int *active = reinterpret_cast<int *>(sc + kScal * kMaxCols);
-    // [0] breakdown, [1] active columns, [2] active probe columns, [3] a bounded wait gave up, [4], [5] CTAs
+    // [0] breakdown (1: a probe column, 2: y), [1] active columns, [2] active probe columns, [3] a bounded wait gave up, [4], [5] CTAs
     // finished, [6] a direction update is pending, [7] which buffer holds the y column's p (YFuse)
     int *flags = active + kMaxCols;
     GP2S_CUDA(c, cudaMemsetAsync(flags, 0, sizeof(int) * 8, c->stream));
@@ -3127,6 +3137,7 @@ gp2s_status cg_run(gp2s_ctx *c, int m, const V *val, const CGBuffers &B, const d
     const int check_every = 8;
     int it = 0;
     int *hcount = reinterpret_cast<int *>(c->hbuf.p);
+    double *hy = reinterpret_cast<double *>(hcount + 8);   // the y column's scalars (trial)
     int mc = m;          // probe columns still iterated; 0 once every probe column has stopped
     // one CG / PCG iteration on the active columns (every argument is fixed for given mc, pcz:
     // the scalars live in device memory), so runs of iterations can be captured into a graph
@@ -3257,7 +3268,8 @@ gp2s_status cg_run(gp2s_ctx *c, int m, const V *val, const CGBuffers &B, const d
             }
         }
         GP2S_CUDA(c, cudaMemcpyAsync(hcount, flags, sizeof(int) * 4, cudaMemcpyDeviceToHost, c->stream));
-        if (rel) GP2S_CUDA(c, cudaMemcpyAsync(hcount + 4, active, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+        if (rel || trial) GP2S_CUDA(c, cudaMemcpyAsync(hcount + 4, active, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+        if (trial) GP2S_CUDA(c, cudaMemcpyAsync(hy, sc, sizeof(double) * kScal, cudaMemcpyDeviceToHost, c->stream));
         GP2S_CUDA(c, cudaStreamSynchronize(c->stream));
         GP2S_TRY(flush_profile(c));
         if (hcount[3]) {
@@ -3273,9 +3285,20 @@ gp2s_status cg_run(gp2s_ctx *c, int m, const V *val, const CGBuffers &B, const d
             GP2S_TRY(replace_y());
             y_back = !rel->done;
         }
+        if (trial && !y_idle && hcount[4]) {
+            const double rate = hy[S_RR] < hy[S_B2] ? std::log(hy[S_RR] / hy[S_B2]) / it : 0.0;
+            const double need = rate < 0.0 ? std::max(0.0, 2.0 * std::log(tol_y) / rate - it) : 1e30;
+            if ((it + need + trial->more) * trial->it_us > trial->budget_us) {
+                GP2S_CUDA(c, cudaMemsetAsync(active, 0, sizeof(int), c->stream));
+                y_idle = true;
+                gr.mc = -1;             // a captured run holds the y column's kernels
+                hcount[1] = hcount[2];
+            }
+        }
         if (hcount[1] == 0 && !y_back) break;
         if (mc > 0 && hcount[2] == 0) mc = 0;   // only the y column is left: y-only kernels
     }
+    if (trial) trial->done = !y_idle && hcount[4] == 0 && !(hcount[0] & 2);
 #undef GP2S_PCZ
 #undef GP2S_PCZ_BJ
 #undef GP2S_PCY
@@ -3290,7 +3313,7 @@ gp2s_status cg_run(gp2s_ctx *c, int m, const V *val, const CGBuffers &B, const d
     int mz = 0;
     for (int cc = 1; cc < k; ++cc) mz = std::max(mz, (int)hs[cc * kScal + S_STEPS]);
     *iters_z = mz;
-    *breakdown = hcount[0] != 0;
+    *breakdown = (hcount[0] & (trial ? 1 : 3)) != 0;
     return GP2S_OK;
 }
 
@@ -3378,16 +3401,34 @@ gp2s_status krylov_columns_solve(gp2s_ctx *c, int m, double tol, int *iters)
 }
 
 // A band matrix (points in one dimension sort into one) factors in far less time than the y column's
-// hundreds to thousands of PCG iterations take on it: n band^2 FP64 multiply-adds, spread over the tile
-// chains that the elimination order leaves independent.  12,452 rows of 168 entries: 1.4 ms against
-// 7,800 iterations of 21 us.  Two-dimensional points already have bands of half the matrix in Morton order
+// hundreds to thousands of PCG iterations take on it: 12,452 rows of 168 entries 1.4 ms against 7,800
+// iterations of 21 us.  Two-dimensional points already have bands of half the matrix in Morton order
 // and stay with PCG (at 20,000 points its 200 iterations cost less than the tiles of the factor).  The
-// limits keep the factor below about 5 ms.  A batch of 24 problems (a third of them 1-D): 386 -> 105 ms.
+// limits keep the factor below about 8 ms.  A batch of 24 problems (a third of them 1-D): 386 -> 105 ms.
 static bool y_direct(const gp2s_ctx *c)
 {
     constexpr int kMaxBand = 512;
     const Assembled &A = c->A;
     return A.band <= kMaxBand && (double)A.n * A.band * A.band <= 2e9;
+}
+
+// What the factor and a y-only iteration cost, in us, from the sizes (one GB300).  The factor: fill, flags and
+// the host's order by rows, tile products by entries times band (65,536 rows of 200 entries 7.0 ms, 180,000 of
+// 40 4.0, 100,000 of 100 5.0, 20,000 of 40 0.8; 7.3, 3.4, 4.2 and 0.6 here).  The iteration: 17.0 us at 2,500
+// rows of 30 entries, 25.6 at 30,000 of 40, 55.9 at 65,000 of 350, 39.0 at 100,000 of 40.
+// A large noise variance makes PCG converge in tens of iterations or fewer, and then the factor loses: 30,000
+// rows of 300 entries, sigma2 = 100, 3.2 ms by PCG against 9.4, 100,000 of 100 2.5 against 6.4; with
+// sigma2 = 1e-3 233 against 25 and 112 against 14.  So where the factor costs more than kDirectAtOnce, y
+// starts beside the probes (TrialY); below that the trial would cost as much as it could save.
+constexpr double kDirectAtOnce = 500.0;
+static TrialY y_trial(const gp2s_ctx *c)
+{
+    const Assembled &A = c->A;
+    TrialY t;
+    t.budget_us = 300.0 + 0.012 * (double)A.n + 3.2e-6 * (double)A.nnz * A.band;
+    t.it_us = 17.0 + 2e-4 * (double)A.n + 1e-6 * (double)A.nnz;
+    t.more = 12;
+    return t;
 }
 
 gp2s_status krylov_solve(gp2s_ctx *c, const double *y_sorted_dev, bool with_probes, int m, int ksteps,
@@ -3477,24 +3518,38 @@ gp2s_status krylov_solve(gp2s_ctx *c, const double *y_sorted_dev, bool with_prob
         }
         return GP2S_OK;
     }
-    // an evaluation without a gradient (training, batches) on a band matrix: the probe columns run their
-    // Lanczos steps beside an idle y column, and y is solved by the tiled Cholesky factor; where that fails
-    // the y column's PCG follows on its own
+    // Reliable updates pay where iterations are dear: each replacement costs a host synchronisation,
+    // about ten launches and up to one check interval of idle y iterations, which a small problem's
+    // cheap restarted refinement undercuts (the 256-problem batch, n <= 65,536: 21 problems/s with
+    // them against 29 without; at n = 1M and 10M they save 13 % and 10 %).
+    const bool reliable = c->reliable_y && n >= c->reliable_min_rows && !y_zero;
+    // an evaluation without a gradient (training, batches) on a band matrix: y is solved by the tiled Cholesky
+    // factor after the probe columns' Lanczos steps, beside which it is idle or on trial; where the factor
+    // fails the y column's PCG follows on its own
     bool direct = mixed && mm > 0 && !y_zero && !c->probes_for_grad && o.precond == 2 && y_direct(c);
     // a matrix that the factorisation refuses is PCG's from the start, beside the probes
     if (direct) GP2S_TRY(exact_fits(c, &direct));
+    TrialY trial = y_trial(c);
     if (direct) {
-        GP2S_CUDA(c, cudaMemsetAsync(r64, 0, sizeof(double) * n, c->stream));
-        GP2S_TRY((cg_run<float, float>(c, mm, c->val32.as<float>(), B, r64, 1.0, tol_z, ksteps, ksteps, rec, o.max_iter,
-                                       &iy, &iz, &brk, nullptr, true)));
+        // (the residual replacements count their convergence in another way)
+        if (trial.budget_us > kDirectAtOnce && !reliable) {
+            GP2S_TRY((cg_run<float, float>(c, mm, c->val32.as<float>(), B, b64, tol_first, tol_z, ksteps, ksteps, rec,
+                                           o.max_iter, &iy, &iz, &brk, nullptr, false, &trial)));
+        } else {
+            GP2S_CUDA(c, cudaMemsetAsync(r64, 0, sizeof(double) * n, c->stream));
+            GP2S_TRY((cg_run<float, float>(c, mm, c->val32.as<float>(), B, r64, 1.0, tol_z, ksteps, ksteps, rec,
+                                           o.max_iter, &iy, &iz, &brk, nullptr, true)));
+        }
         if (brk) return set_err(c, GP2S_EBREAKDOWN, "CG breakdown (p^T A p <= 0 or NaN)");
+        res->iters_probes = iz;
+        c->have_probes = true;
+        c->probe_iters = iz;
+    }
+    if (direct && !trial.done) {
         double ld = 0.0, relres = 0.0;
         const gp2s_status st = exact_logdet_solve(c, y_sorted_dev, &ld);
         if (st == GP2S_OK) GP2S_TRY(y_residual(c, y_sorted_dev, &relres));
         else if (st != GP2S_ENOTPD && st != GP2S_ENOMEM) return st;
-        res->iters_probes = iz;
-        c->have_probes = true;
-        c->probe_iters = iz;
         if (st == GP2S_OK && relres <= o.tol_refine) {
             res->iters_y = res->outer = 0;
             res->relres = relres;
@@ -3516,12 +3571,9 @@ gp2s_status krylov_solve(gp2s_ctx *c, const double *y_sorted_dev, bool with_prob
     ru.y_sorted = y_sorted_dev;
     ru.tol_refine = o.tol_refine;
     ru.delta = c->reliable_delta;
-    // Reliable updates pay where iterations are dear: each replacement costs a host synchronisation,
-    // about ten launches and up to one check interval of idle y iterations, which a small problem's
-    // cheap restarted refinement undercuts (the 256-problem batch, n <= 65,536: 21 problems/s with
-    // them against 29 without; at n = 1M and 10M they save 13 % and 10 %).
-    const bool reliable = c->reliable_y && n >= c->reliable_min_rows && !y_zero;
-    if (mixed)
+    if (trial.done) {
+        // y converged beside the probes
+    } else if (mixed)
         GP2S_TRY((cg_run<float, float>(c, my, c->val32.as<float>(), B, b64, tol_first, tol_z, my > 0 ? ksteps : 0,
                                        ksteps, my > 0 ? rec : nullptr, o.max_iter, &iy, &iz, &brk,
                                        reliable ? &ru : nullptr, y_zero)));

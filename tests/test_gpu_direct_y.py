@@ -64,3 +64,31 @@ def test_a_matrix_that_the_factorisation_refuses_keeps_y_beside_the_probes(gp, m
     assert info["quad"] == with_grad["quad"]
     assert info["iters_probes"] == free["iters_probes"] and info["logdet"] == pytest.approx(free["logdet"], rel=1e-12)
     assert info["quad"] == pytest.approx(free["quad"], rel=1e-7)
+
+
+@pytest.mark.parametrize("n,row,sigma2", [(30_000, 300, 100.0), (100_000, 100, 100.0), (65_536, 200, 10.0)])
+def test_a_system_of_few_iterations_is_not_factored(gp, n, row, sigma2):
+    """A large noise variance leaves PCG a handful of iterations, beside the probes' steps, where the factor of
+    these bands takes 4 to 7 ms.  The evaluation with the gradient, which never factors, takes the same steps."""
+    X, y, hyper = _line(n, row, sigma2)
+    h = gp.Hyper(**hyper)
+    opts = gp.default_opts(logdet=gp.LOGDET_SLQ, probes=16, lanczos_steps=100, seed=3, tol_probe=1.0)
+    ctx = gp.Context(0)
+    info = ctx.lml(X, y, h, opts)[1]
+    with_grad = ctx.lml_grad(X, y, h, opts)[2]
+    assert 0 < info["iters_y"] <= 60 and info["iters_y"] == with_grad["iters_y"]
+    assert info["quad"] == with_grad["quad"] and info["relres"] == with_grad["relres"] <= 1e-8
+    assert info["logdet"] == with_grad["logdet"] and info["iters_probes"] == with_grad["iters_probes"]
+
+
+@pytest.mark.parametrize("n,row,probes,steps", [(20_000, 40, 16, 100), (20_000, 40, 48, 7), (65_000, 200, 64, 20), (9000, 300, 32, 8)])
+def test_a_y_column_given_up_leaves_the_probes_as_they_are(gp, n, row, probes, steps):
+    """y starts beside the probes, does not converge and is left to the factor: at the check after eight
+    steps, with the probes at their end or on their way.  Their records are those of the log-determinant
+    alone, whose y column is idle from the first step."""
+    X, y, hyper = _line(n, row, 1e-3)
+    opts = gp.default_opts(logdet=gp.LOGDET_SLQ, probes=probes, lanczos_steps=steps, seed=3)
+    ctx = gp.Context(0)
+    info = ctx.lml(X, y, gp.Hyper(**hyper), opts)[1]
+    assert info["iters_y"] == 0 and info["relres"] <= 1e-10
+    assert ctx.logdet()[0] == pytest.approx(info["logdet"], rel=1e-13)
