@@ -55,6 +55,14 @@ gp2s_status ensure(gp2s_ctx *c, DevBuf &b, size_t bytes)
     return GP2S_OK;
 }
 
+void release(gp2s_ctx *c, DevBuf &b)
+{
+    if (b.p) cudaFree(b.p);
+    c->mem_in_use -= b.bytes;
+    b.p = nullptr;
+    b.bytes = 0;
+}
+
 gp2s_status smem_attr(gp2s_ctx *c, const void *func, size_t smem)
 {
     // The attribute belongs to the function on this device, shared by every context and host

@@ -747,4 +747,12 @@ gp2s_status exact_logdet_solve(gp2s_ctx *c, const double *y_sorted_dev, double *
     return GP2S_OK;
 }
 
+void exact_release(gp2s_ctx *c)
+{
+    release(c, c->dense);
+    release(c, c->chol_ints);
+    c->chol_plan_valid = false;
+    c->have_exact = false;
+}
+
 }  // namespace gp2s

@@ -206,6 +206,7 @@ namespace gp2s {
 gp2s_status set_err(gp2s_ctx *c, gp2s_status st, const std::string &msg);
 gp2s_status cuda_err(gp2s_ctx *c, cudaError_t e, const char *where);
 gp2s_status ensure(gp2s_ctx *c, DevBuf &b, size_t bytes);
+void release(gp2s_ctx *c, DevBuf &b);
 gp2s_status ensure_host(gp2s_ctx *c, HostPinned &b, size_t bytes);
 // Raise a kernel's dynamic shared-memory limit to at least smem bytes (thread-safe, grow-only).
 gp2s_status smem_attr(gp2s_ctx *c, const void *func, size_t smem);
@@ -269,6 +270,8 @@ gp2s_status krylov_columns_solve(gp2s_ctx *c, int m, double tol, int *iters);
 gp2s_status exact_fits(gp2s_ctx *c, bool *fits);
 // log|Ah| by tiled Cholesky and, with y_sorted_dev, a = A^{-1} y in vec64 slot 3 (cholesky.cu).
 gp2s_status exact_logdet_solve(gp2s_ctx *c, const double *y_sorted_dev, double *logdet_hat);
+// Give back the factor's buffers and the plan (the stream's work on them has finished).
+void exact_release(gp2s_ctx *c);
 // Reductions used by several stages
 gp2s_status sum_log_diag(gp2s_ctx *c, double *out_host);
 gp2s_status dot_f64(gp2s_ctx *c, const double *a, const double *b, int64_t n, double *out_host);

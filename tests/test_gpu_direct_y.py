@@ -92,3 +92,53 @@ def test_a_y_column_given_up_leaves_the_probes_as_they_are(gp, n, row, probes, s
     info = ctx.lml(X, y, gp.Hyper(**hyper), opts)[1]
     assert info["iters_y"] == 0 and info["relres"] <= 1e-10
     assert ctx.logdet()[0] == pytest.approx(info["logdet"], rel=1e-13)
+
+
+def _least_limit(gp, monkeypatch, call):
+    """The least GP2S_MEM_LIMIT, to 1 KB, under which `call` succeeds on a context of its own."""
+    lo, hi = 0, 1 << 17
+    while hi - lo > 1:
+        mid = (lo + hi) // 2
+        monkeypatch.setenv("GP2S_MEM_LIMIT", str(mid << 10))
+        try:
+            call(gp.Context(0))
+            hi = mid
+        except gp.GP2SError as e:
+            assert e.status == gp.ENOMEM
+            lo = mid
+    monkeypatch.setenv("GP2S_MEM_LIMIT", str(hi << 10))
+    return hi << 10
+
+
+@pytest.mark.parametrize("n,row,steps", [(300, 30, 20), (500, 60, 3), (501, 200, 100)])
+def test_a_factor_without_room_leaves_y_to_pcg(gp, monkeypatch, n, row, steps):
+    """Under the least limit that the evaluation itself fits in, the factor's buffers are refused after the
+    probes have run: y's PCG follows on its own, with the same probe records and the same results."""
+    X, y, hyper = _line(n, row, 1e-3)
+    h = gp.Hyper(**hyper)
+    opts = gp.default_opts(logdet=gp.LOGDET_SLQ, probes=16, lanczos_steps=steps, seed=3)
+    free = gp.Context(0).lml(X, y, h, opts)[1]
+    assert free["iters_y"] == 0
+    limit = _least_limit(gp, monkeypatch, lambda c: c.lml(X, y, h, opts))
+    assert limit >= 8 * n * n          # the factorisation is tried
+    ctx = gp.Context(0)
+    for _ in range(2):
+        info = ctx.lml(X, y, h, opts)[1]
+        assert info["iters_y"] > 0 and info["relres"] <= 1e-8
+        assert info["iters_probes"] == free["iters_probes"]
+        assert info["logdet"] == pytest.approx(free["logdet"], rel=1e-13)
+        assert info["quad"] == pytest.approx(free["quad"], rel=1e-7)
+
+
+@pytest.mark.parametrize("n", [300, 500])
+def test_a_factor_under_a_limit_takes_no_room_from_later_calls(gp, monkeypatch, n):
+    """A larger call (four times the probes, with the gradient) that fits the limit on a fresh context still
+    fits after an evaluation whose y solve took the factor."""
+    X, y, hyper = _line(n, 30, 1e-3)
+    h = gp.Hyper(**hyper)
+    small = gp.default_opts(logdet=gp.LOGDET_SLQ, probes=16, lanczos_steps=20, seed=3)
+    large = gp.default_opts(logdet=gp.LOGDET_SLQ, probes=64, lanczos_steps=20, seed=3)
+    _least_limit(gp, monkeypatch, lambda c: c.lml_grad(X, y, h, large))
+    ctx = gp.Context(0)
+    assert ctx.lml(X, y, h, small)[1]["iters_y"] == 0
+    ctx.lml_grad(X, y, h, large)
