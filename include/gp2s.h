@@ -45,7 +45,9 @@ typedef enum {
     GP2S_EBREAKDOWN = 5,  /* CG breakdown: p^T A p <= 0 or NaN while the column's residual is still
                              above the rounding level of its precision (a column whose residual has
                              reached it just stops: its Krylov space is exhausted) */
-    GP2S_ETIMEOUT = 6,    /* reserved: a bounded device-side wait gave up */
+    GP2S_ETIMEOUT = 6,    /* a bounded device-side wait gave up: a bulk copy of a Krylov kernel (gp2s_solve,
+                             gp2s_logdet, gp2s_lml*, gp2s_posterior) or a tile of the exact
+                             factorisation (GP2S_LOGDET_EXACT) did not complete in seconds */
     GP2S_EOVERFLOW = 7,   /* nnz would exceed 2^31 - 1 (int32 column / row-pointer limit) */
     GP2S_ENOTPD = 8,      /* A not positive definite (zero diagonal, Cholesky pivot <= 0) */
     GP2S_ENOTREADY = 9    /* the call needs an earlier gp2s_assemble / gp2s_solve on this context */

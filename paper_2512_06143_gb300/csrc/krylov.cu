@@ -3549,7 +3549,7 @@ gp2s_status krylov_solve(gp2s_ctx *c, const double *y_sorted_dev, bool with_prob
         double ld = 0.0, relres = 0.0;
         const gp2s_status st = exact_logdet_solve(c, y_sorted_dev, &ld);
         if (st == GP2S_OK) GP2S_TRY(y_residual(c, y_sorted_dev, &relres));
-        else if (st != GP2S_ENOTPD && st != GP2S_ENOMEM) return st;
+        else if (st != GP2S_ENOTPD && st != GP2S_ENOMEM && st != GP2S_ETIMEOUT) return st;
         // under a limit the factor's buffers leave the room that they found to the calls that follow
         if (c->mem_limit) exact_release(c);
         if (st == GP2S_OK && relres <= o.tol_refine) {

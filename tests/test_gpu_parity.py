@@ -312,6 +312,25 @@ def test_tiled_cholesky_at_tile_edges(gp, ctx, n, d, r):
     assert info["relres"] <= 1e-12      # the residual is formed from this call's right-hand side and solution
 
 
+@pytest.mark.parametrize("n,d,row,r", [(12_000, 2, 60, None), (9_001, 3, 60, None), (4_097, 2, 0, 3.0)])
+def test_tiled_cholesky_with_much_fill(gp, ctx, n, d, row, r):
+    """Larger tile graphs than the ones above (2-D, 3-D with its heavy fill, every tile present): long lists of
+    products per tile, more tasks than resident CTAs.  The reference is the dense Cholesky factor of the same
+    matrix in FP64; n rounding errors of 1.1e-16 on each of n pivots' logarithms stay below 1e-11 n."""
+    w = W.random_small(720 + n, n, d, L=3, sigma2=1e-2, r=r)
+    if r is None:
+        w["hyper"]["r"] *= (row / 30.0) ** (1.0 / d)
+    opts = gp.default_opts(precision=gp.PREC_FP64, logdet=gp.LOGDET_EXACT)
+    _, info = ctx.lml(w["X"], w["y"], gp.Hyper(**w["hyper"]), opts)
+    assert info["relres"] <= 1e-12
+    c = ctx.csr()
+    A = torch.zeros(n, n, dtype=torch.float64, device="cuda")
+    rows = torch.repeat_interleave(torch.arange(n, device="cuda"), c["rowptr"].diff())
+    A[rows, c["col"].long()] = c["val64"]
+    ref = 2.0 * torch.linalg.cholesky(A).diagonal().log().sum().item()
+    assert ctx.logdet()[2]["logdet_hat"] == pytest.approx(ref, abs=1e-11 * n)
+
+
 @pytest.mark.parametrize("steps,rel", [(1, 1e-9), (2, 1e-9), (33, 1e-9), (257, 1e-6), (300, 1e-6)])
 def test_slq_quadrature_matches_the_oracle_eigensolve(gp, ctx, steps, rel):
     """The quadrature of log T without its eigen-decomposition against the oracle's Gauss quadrature, in
