@@ -2489,8 +2489,6 @@ k_pc_step(int64_t n, int m, int64_t nblk, int gz, const float *__restrict__ Minv
 // ---------------------------------------------------------------------------------------------
 constexpr int kPPProducers = 256, kPPConsumers = 128;
 constexpr int kPPThreads = kPPProducers + kPPConsumers;
-// CTAs per SM: 64-row blocks and 32 columns leave room for two (101 KB of stages each)
-template <int SB, int M> constexpr int pp_ctas = (SB == 64 && M == 32) ? 2 : 1;
 
 // two stages of (M^{-1} block, residual block), the y column's two staged residual blocks (WY), the
 // two mbarriers
@@ -2508,7 +2506,7 @@ size_t pp_smem()
 // consecutive 64 x 64 blocks of M^{-1}, contiguous in memory, and each tile multiplies within its
 // own block).
 template <int BJ, int SB, int M, bool WY>
-__global__ void __launch_bounds__(kPPThreads, (pp_ctas<SB, M>))
+__global__ void __launch_bounds__(kPPThreads, 1)
 k_pc_probe(int64_t n, int64_t nblk, const float *__restrict__ Minv32, float *__restrict__ rz,
            const float *__restrict__ qz, float *__restrict__ zz, const double *__restrict__ sc,
            double *__restrict__ part_rz, double *__restrict__ part_rr, int pstride, int *__restrict__ err,
@@ -2524,9 +2522,12 @@ k_pc_probe(int64_t n, int64_t nblk, const float *__restrict__ Minv32, float *__r
     // tiles of twice the threads took 3 for 16, and shared-memory loads and FMAs of this size do not
     // overlap: their times added up), 8 x 4 with 32.  The 8 columns are two runs of 4, M / 2 apart, so that
     // the lanes' loads stay contiguous.  (Scalar FMAs in place of the packed ones: 446 against 402 us at 1M rows.)
-    // Per launch, 64-row blocks at 100,000 rows: 64 columns 49.9 us with 8 x 4 tiles and the y column, 32.8
-    // without y; 32 columns with y 40.4 -> 28.6 (two CTAs per SM, the y column's sums by trees).
-    // 128-row blocks at 1M rows: 403 us before and after, bound by the consumers' FMAs and loads.
+    // Per launch, 64-row blocks: 64 columns at 100,000 rows 49.9 us with 8 x 4 tiles and the y column, 32.8
+    // without y; 32 columns with y 40.9 -> 23.6 us at 100,000 rows, 177 -> 159 at 1M, 1208 -> 1186 at 8M (the y
+    // column's sums by trees, a tile for every consumer).  One CTA per SM: two fit the shared memory of 64-row
+    // blocks with 32 columns, but at 80 registers a thread they spill (28.1, 180 and 1342 us).
+    // 128-row blocks at 1M rows: 403 us (64 columns; 400 with 8 x 4 tiles), bound by the consumers' FMAs and
+    // loads, and 236 (32 columns; 262).
     constexpr int NP = kPPProducers, NC = kPPConsumers;
     constexpr int CG = M / 4;                  // column groups of four (producers)
     constexpr int NF4 = BJ * M / 4;            // float4 per residual block
@@ -3070,7 +3071,7 @@ gp2s_status cg_run(gp2s_ctx *c, int m, const V *val, const CGBuffers &B, const d
     const bool pc_async = pc_avail && c->pc_async && (m == 32 || m == 64) &&
                           (bjz == 128 || (bjz == 64 && c->pc_async64));
     const int64_t nstage = ceil_div(n, (int64_t)128);   // the bulk-copy kernel's 128-row stages
-    const int pga = (int)std::min<int64_t>((int64_t)c->num_sms * (bjz == 64 && m == 32 ? pp_ctas<64, 32> : 1), nstage);
+    const int pga = (int)std::min<int64_t>(c->num_sms, nstage);
     int *dev_err = flags + 3;
     // the y column's PCG update joins the probe group's step when both use the same factors
     const bool pc_fuse_y = pcy && bjy == bjz && c->pc_fuse_y;
