@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "gp2s_cholesky.cuh"
+#include "gp2s_kernel_math.cuh"
 
 namespace gp2s {
 
@@ -66,21 +67,6 @@ __device__ __forceinline__ bool chol_positive(double d)
 {
     const int hi = __double2hiint(d);
     return hi < 0x7ff00000 && (hi > 0 || (hi == 0 && __double2loint(d) != 0));
-}
-
-// 1 / d for a usable pivot: the FP32 reciprocal (relative error e below 2^-20) and one cubic step
-// r (1 + e + e^2), three dependent FP64 operations instead of a full division's chain.  The conversions
-// to FP32 and back move the exponent and the upper 23 bits of the mantissa with integer operations, as
-// converting is FP64 work too; outside 2^-100 .. 2^100 the division itself.
-__device__ __forceinline__ double chol_rcp(double d)
-{
-    const int hi = __double2hiint(d), lo = __double2loint(d);
-    if (hi < ((1023 - 100) << 20) || hi >= ((1023 + 100) << 20)) return 1.0 / d;
-    const float f = __int_as_float(((hi - ((1023 - 127) << 20)) << 3) | (int)((unsigned)lo >> 29));
-    const int rf = __float_as_int(1.0f / f);
-    const double r = __hiloint2double((rf >> 3) + ((1023 - 127) << 20), rf << 29);
-    const double e = fma(-d, r, 1.0);
-    return fma(r, fma(e, e, e), r);
 }
 
 template <bool ALL> struct CholMap;
@@ -298,7 +284,7 @@ k_chol(const CholArgs a)
                     if (8 * wid + 7 > c) {
                         double d = colbuf[c & 1][c];
                         if (!chol_positive(d)) d = 1.0;
-                        const double w = colbuf[c & 1][r4] * chol_rcp(d);
+                        const double w = colbuf[c & 1][r4] * rcp_pos(d);
 #pragma unroll
                         for (int m = 0; m < 8; ++m)
                             if (4 * m > c || (4 * m + 3 > c && q4 + 4 * m > c)) v[m] = fma(-w, colbuf[c & 1][q4 + 4 * m], v[m]);

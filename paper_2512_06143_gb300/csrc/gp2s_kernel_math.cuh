@@ -68,8 +68,10 @@ __device__ __forceinline__ T wendland_dt_over_t(int kind, int d, T t)
 // Square root of q >= 0 in six FP64 operations: the FP32 reciprocal root y of q (its exponent and upper
 // mantissa bits moved to FP32 and back by integer operations, since conversions are FP64 work), one coupled
 // Newton step for g ~ sqrt(q) and h ~ 1 / (2 sqrt(q)) (Goldschmidt's iteration), and the residual
-// correction g + (q - g^2) h, whose own error is below 2^-80 relative: the rounding of the last
-// operation remains.  Zero, and values outside 2^-100 .. 2^100, take sqrt().
+// correction g + (q - g^2) h.  y is off by less than 2^-21, g and h by 2^-42, so before its last rounding
+// the result is off by less than 2^-80: it is the correctly rounded root unless that root lies
+// within 2^-80 of the middle between two doubles (one q in 2^26), and then it may be its neighbour.  Zero, and
+// values outside 2^-100 .. 2^100, take sqrt().
 __device__ __forceinline__ double sqrt_pos(double q)
 {
     const int hi = __double2hiint(q), lo = __double2loint(q);
@@ -82,6 +84,21 @@ __device__ __forceinline__ double sqrt_pos(double q)
     const double e = fma(-g0, h0, 0.5);
     const double g = fma(g0, e, g0), h = fma(h0, e, h0);
     return fma(fma(-g, g, q), h, g);
+}
+
+// 1 / d for a positive finite d in three dependent FP64 operations instead of a full division's chain: the
+// FP32 reciprocal r (the same bit moves; 1 - d r = e below 2^-22) and one step of Chebyshev's third-order
+// iteration, r (1 + e + e^2).  Off by less than 2^-65 before the last rounding: within an ulp of the
+// quotient, and equal to it but for one d in some thousands.  Outside 2^-100 .. 2^100 the division itself.
+__device__ __forceinline__ double rcp_pos(double d)
+{
+    const int hi = __double2hiint(d), lo = __double2loint(d);
+    if (hi < ((1023 - 100) << 20) || hi >= ((1023 + 100) << 20)) return 1.0 / d;
+    const float f = __int_as_float(((hi - ((1023 - 127) << 20)) << 3) | (int)((unsigned)lo >> 29));
+    const int rf = __float_as_int(1.0f / f);
+    const double r = __hiloint2double((rf >> 3) + ((1023 - 127) << 20), rf << 29);
+    const double e = fma(-d, r, 1.0);
+    return fma(r, fma(e, e, e), r);
 }
 #endif
 
