@@ -496,6 +496,25 @@ def test_block_jacobi_factors_at_block_edges(gp, ctx, bj, n):
         assert info["iters"] <= 4 * (info["outer"] + 1)
 
 
+@pytest.mark.parametrize("bj", [64, 128])
+@pytest.mark.parametrize("blocks,rest", [(2, 0), (2, 1), (3, 37), (8, 63), (160, 5)])
+def test_block_jacobi_factors_of_every_block(gp, ctx, bj, blocks, rest):
+    """Points in one dimension in clusters of a block's rows, further apart than the support: M is A again, block
+    by block, the last one ragged, and the few-step bound of a single block holds for all of them.  A block
+    that is wrong, or taken from other rows, needs more."""
+    n, r = bj * blocks + rest, 1e-3
+    w = W.random_small(840 + n, n, 1, L=3, sigma2=0.1, r=r)
+    rng = np.random.default_rng(n)
+    w["X"][:, 0] = (np.arange(n) // bj) * 4 * r + 0.8 * r * rng.random(n)
+    order = rng.permutation(n)
+    h = gp.Hyper(**w["hyper"])
+    info = ctx.assemble(w["X"][order], h, gp.default_opts(precond=2, bj_block=bj))
+    assert info["nnz"] == bj * bj * blocks + rest * rest
+    _, s = ctx.solve(w["y"][order])
+    assert s["relres"] <= 1e-8
+    assert s["iters"] <= 4 * (s["outer"] + 1)
+
+
 def test_autograd_function(gp, ctx):
     w = W.random_small(303, 3000, 2, L=2, sigma2=1e-3)
     h = gp.Hyper(**w["hyper"])
