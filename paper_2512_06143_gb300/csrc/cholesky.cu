@@ -186,6 +186,7 @@ k_chol(const CholArgs a)
         if (s_task >= a.ntasks) break;
         const int4 task = Map::task(a, s_task);
         const int j = task.z;
+        const int o = Map::origin(a, j) * kCT, rows = min(kCT, a.n - o);   // rows of the matrix in tile row j
         if (task.x != CT_FACTOR && !a.solve) continue;
         if (task.x == CT_FACTOR) {
             const int i = task.y;
@@ -278,6 +279,7 @@ k_chol(const CholArgs a)
                 // L D L^T by columns (one reciprocal per column), scaled to L L^T at the end
 #pragma unroll
                 for (int c = 0; c < kCT; ++c) {
+                    if (c >= rows) break;            // identity rows: nothing below their pivots
                     if (q4 == (c & 3)) colbuf[c & 1][r4] = v[c >> 2];
                     __syncthreads();
                     // rows up to c are finished (a warp holds eight rows)
@@ -340,7 +342,6 @@ k_chol(const CholArgs a)
         } else {
             // one block of the forward (L y = b) or backward (L^T x = y) solve
             const bool fw = task.x == CT_FORWARD;
-            const int o = Map::origin(a, j) * kCT;
             double acc = 0.0;                       // row / column r4's sum over the lanes' q4
             if (fw) {
                 const int kb = Map::row_begin(a, j), ke = Map::row_end(a, j);
@@ -384,7 +385,7 @@ k_chol(const CholArgs a)
                 v -= vec[lane];
                 if (fw) {
 #pragma unroll 8
-                    for (int c = 0; c < kCT; ++c) {
+                    for (int c = 0; c < rows; ++c) {
                         const double x = __shfl_sync(0xffffffffu, v * inv, c);
                         if (lane == c) v = x;
                         else if (lane > c) v = fma(-x, Bs_[lane][c], v);
@@ -392,7 +393,7 @@ k_chol(const CholArgs a)
                     a.yv[j * kCT + lane] = v;
                 } else {
 #pragma unroll 8
-                    for (int c = kCT - 1; c >= 0; --c) {
+                    for (int c = rows - 1; c >= 0; --c) {
                         const double x = __shfl_sync(0xffffffffu, v * inv, c);
                         if (lane == c) v = x;
                         else if (lane < c) v = fma(-x, Bs_[c][lane], v);
@@ -640,15 +641,18 @@ static gp2s_status chol_plan(gp2s_ctx *c)
     // an entry `band` below the diagonal lies at most ceil(band / kCT) tiles below it
     const int nt = (int)ceil_div(n, kCT), words = std::max(1, (int)ceil_div(ceil_div(c->A.band, kCT), 32));
     const size_t nbits = (size_t)nt * words;
-    GP2S_TRY(ensure(c, c->chol_ints, sizeof(unsigned) * nbits));
-    GP2S_CUDA(c, cudaMemsetAsync(c->chol_ints.p, 0, sizeof(unsigned) * nbits, c->stream));
-    const unsigned gb = (unsigned)std::min<int64_t>(ceil_div(n * 32, 256), 152 * 16);
-    k_chol_bits<<<gb, 256, 0, c->stream>>>(c->rowptr.as<int32_t>(), c->col.as<int32_t>(), n, words,
-                                           c->chol_ints.as<unsigned>());
-    GP2S_LAUNCH(c);
     std::vector<uint32_t> low(nbits);
-    GP2S_CUDA(c, cudaMemcpyAsync(low.data(), c->chol_ints.p, sizeof(unsigned) * nbits, cudaMemcpyDeviceToHost, c->stream));
-    GP2S_CUDA(c, cudaStreamSynchronize(c->stream));
+    if (nt > 1) {                                     // (one tile has no neighbours)
+        GP2S_TRY(ensure(c, c->chol_ints, sizeof(unsigned) * nbits));
+        GP2S_CUDA(c, cudaMemsetAsync(c->chol_ints.p, 0, sizeof(unsigned) * nbits, c->stream));
+        const unsigned gb = (unsigned)std::min<int64_t>(ceil_div(n * 32, 256), 152 * 16);
+        k_chol_bits<<<gb, 256, 0, c->stream>>>(c->rowptr.as<int32_t>(), c->col.as<int32_t>(), n, words,
+                                               c->chol_ints.as<unsigned>());
+        GP2S_LAUNCH(c);
+        GP2S_CUDA(c, cudaMemcpyAsync(low.data(), c->chol_ints.p, sizeof(unsigned) * nbits, cudaMemcpyDeviceToHost,
+                                     c->stream));
+        GP2S_CUDA(c, cudaStreamSynchronize(c->stream));
+    }
     CholPlan P;
     chol_order(nt, words, low, P);
     // one upload: tasks (16-byte aligned), then the int lists
