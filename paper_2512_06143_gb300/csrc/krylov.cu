@@ -490,8 +490,11 @@ __global__ void k_scal_beta(const double *__restrict__ part, const double *__res
 // With DIR the direction kernel goes as well: beta leaves its update pending (flags[6]), and the next SpMV
 // gathers z + beta p (k_direction's FMA) in place of p, the owner of a row writing the new p into the
 // other of two buffers (flags[7] says which one holds p now).  Two gathers per entry instead of one and a
-// launch: taken up to kYDirRows rows, where both vectors (512 KB) stay close to the SMs; at 100,000 rows and
-// more the iteration is bound by the matrix and the launch no longer shows.
+// launch: taken up to kYDirRows rows, since a launch costs about 1.5 us and the second gather grows with the
+// rows.  Launches apart -> this, us an iteration with its share of the solve: 3,000 rows of 35 entries 22.4 ->
+// 21.7, of 80 21.0 -> 19.8; 20,000 rows of 20, 38, 90 and 173 entries 30.5 -> 28.9, 26.4 -> 26.0, 26.0 ->
+// 26.2, 24.4 -> 24.5; 40,000 of 20, 38, 92, 177 31.6 -> 32.1, 28.3 -> 29.2, 27.9 -> 28.5, 31.1 -> 32.4;
+// 65,000 of 39 33.1 -> 35.0; 100,003 of 41 37.5 -> 40.4; 200,000 of 41 62.3 -> 71.5.
 // An iteration of six launches took 21.4 us at n = 2,500 (1-D), 24.3 us at 12,452 rows of 168 entries; with
 // the scalars fused 18.6 and 22.9 us, with the direction too 17.0 and 21.4 us.
 struct YFuse {
@@ -500,7 +503,7 @@ struct YFuse {
     double lucky;
     int dir = 0;               // the direction update is left to the next SpMV
 };
-constexpr int64_t kYDirRows = 1 << 16;
+constexpr int64_t kYDirRows = 1 << 14;
 
 // Called by every thread of the CTA once its partial sums are written (by thread 0): true in the CTA that
 // finishes last.
