@@ -14,9 +14,10 @@ template <class T>
 __device__ __forceinline__ T wendland(int kind, int d, T t)
 {
     if constexpr (sizeof(T) == 8) {
-        // read off the high word: an FP64 comparison costs as much as an addition
+        // read off the high word: an FP64 comparison costs as much as an addition.  NaN is outside the
+        // support whatever its sign (inf - inf has the sign bit set)
         const int hi = __double2hiint((double)t);
-        if (hi >= 0x3ff00000) return T(0);
+        if (hi >= 0x3ff00000 || (unsigned)hi > 0xfff00000u) return T(0);
         if (hi < 0) t = T(0);
     } else {
         if (!(t < T(1))) return T(0);

@@ -91,6 +91,24 @@ def test_noalloc_at_tile_edges(gp, n):
     assert out == pytest.approx([e["lml"], e["quad"], e["logdet"]], rel=1e-10, abs=1e-10 * n)
 
 
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+def test_noalloc_with_a_coordinate_that_is_not_finite(gp, bad):
+    """A point whose distances are NaN lies outside every support, its own included: it leaves sigma^2 on the
+    diagonal and the other points as they are.  (Inf - inf is a NaN with its sign bit set.)"""
+    import oracle
+    w = W.random_small(450, 40, 2, L=2, sigma2=1e-2, r=0.3, w0=0.5)
+    h = gp.Hyper(**w["hyper"])
+    X = w["X"].copy()
+    X[7, 1] = bad
+    st, out = _noalloc(gp, torch.tensor(X, device="cuda"), torch.tensor(w["y"], device="cuda"), h)
+    assert st == gp.OK
+    rest = np.arange(40) != 7
+    e = oracle.lml_exact(w["X"][rest], w["y"][rest], oracle.Hyper(**w["hyper"]))
+    quad, logdet = e["quad"] + w["y"][7] ** 2 / h.sigma2, e["logdet"] + np.log(h.sigma2)
+    lml = -0.5 * quad - 0.5 * logdet - 20 * np.log(2 * np.pi)
+    assert out == pytest.approx([lml, quad, logdet], rel=1e-9)
+
+
 def test_noalloc_rejects_sizes_beyond_the_limit(gp):
     w = W.random_small(403, 513, 2)
     h = gp.Hyper(**w["hyper"])
