@@ -186,7 +186,12 @@ k_chol(const CholArgs a)
         if (s_task >= a.ntasks) break;
         const int4 task = Map::task(a, s_task);
         const int j = task.z;
-        const int o = Map::origin(a, j) * kCT, rows = min(kCT, a.n - o);   // rows of the matrix in tile row j
+        // rows of the matrix in tile row j: the identity rows past them have nothing to compute.  A full tile
+        // pays for a test every 8 pivots and every 8 steps of a solve: the allocation-free call at 1, 2, 16, 33 and 100
+        // points 58.6 -> 44.6, 60.2 -> 46.0, 62.8 -> 54.2, 105.7 -> 91.7, 184.9 -> 172.0 us, at 512 662.8 -> 663.8.  With a
+        // test per row, and the origin's load for it, 40.2, 43.8, 55.1, 87.4, 170.6, but 669.7 at 512 and up to 2 % of
+        // the exact evaluations of 1,000 to 4,000 points; every 4 steps and after 1, 2 and 4 pivots was no better there.
+        const int rows = j == a.last ? a.n - (a.nt - 1) * kCT : kCT;
         if (task.x != CT_FACTOR && !a.solve) continue;
         if (task.x == CT_FACTOR) {
             const int i = task.y;
@@ -279,7 +284,7 @@ k_chol(const CholArgs a)
                 // L D L^T by columns (one reciprocal per column), scaled to L L^T at the end
 #pragma unroll
                 for (int c = 0; c < kCT; ++c) {
-                    if (c >= rows) break;            // identity rows: nothing below their pivots
+                    if (c % 8 == 0 && c >= rows) break;
                     if (q4 == (c & 3)) colbuf[c & 1][r4] = v[c >> 2];
                     __syncthreads();
                     // rows up to c are finished (a warp holds eight rows)
@@ -342,6 +347,7 @@ k_chol(const CholArgs a)
         } else {
             // one block of the forward (L y = b) or backward (L^T x = y) solve
             const bool fw = task.x == CT_FORWARD;
+            const int o = Map::origin(a, j) * kCT;
             double acc = 0.0;                       // row / column r4's sum over the lanes' q4
             if (fw) {
                 const int kb = Map::row_begin(a, j), ke = Map::row_end(a, j);
@@ -384,19 +390,23 @@ k_chol(const CholArgs a)
                 if (fw && a.bh && o + lane < a.n) a.bh[o + lane] = v;
                 v -= vec[lane];
                 if (fw) {
-#pragma unroll 8
-                    for (int c = 0; c < rows; ++c) {
-                        const double x = __shfl_sync(0xffffffffu, v * inv, c);
-                        if (lane == c) v = x;
-                        else if (lane > c) v = fma(-x, Bs_[lane][c], v);
+                    for (int c0 = 0; c0 < rows; c0 += 8) {
+#pragma unroll
+                        for (int c = c0; c < c0 + 8; ++c) {
+                            const double x = __shfl_sync(0xffffffffu, v * inv, c);
+                            if (lane == c) v = x;
+                            else if (lane > c) v = fma(-x, Bs_[lane][c], v);
+                        }
                     }
                     a.yv[j * kCT + lane] = v;
                 } else {
-#pragma unroll 8
-                    for (int c = rows - 1; c >= 0; --c) {
-                        const double x = __shfl_sync(0xffffffffu, v * inv, c);
-                        if (lane == c) v = x;
-                        else if (lane < c) v = fma(-x, Bs_[c][lane], v);
+                    for (int c0 = (rows - 1) / 8 * 8; c0 >= 0; c0 -= 8) {
+#pragma unroll
+                        for (int c = c0 + 7; c >= c0; --c) {
+                            const double x = __shfl_sync(0xffffffffu, v * inv, c);
+                            if (lane == c) v = x;
+                            else if (lane < c) v = fma(-x, Bs_[c][lane], v);
+                        }
                     }
                     a.xv[j * kCT + lane] = v;
                     if (o + lane < a.n) {
@@ -671,6 +681,7 @@ static gp2s_status chol_plan(gp2s_ctx *c)
     c->chol_nt = nt;
     c->chol_ntiles = (int)P.rowpos.size();
     c->chol_ntasks = (int)P.tasks.size();
+    c->chol_last = P.pos[nt - 1];
     c->chol_plan_valid = true;
     return GP2S_OK;
 }
@@ -684,6 +695,7 @@ gp2s_status exact_logdet_solve(gp2s_ctx *c, const double *y_sorted_dev, double *
     a.nt = c->chol_nt;
     a.ntiles = c->chol_ntiles;
     a.n = (int)n;
+    a.last = c->chol_last;
     a.solve = y_sorted_dev != nullptr;
     a.ntasks = c->chol_ntasks;
     a.tasks = c->chol_ints.as<int4>();

@@ -16,6 +16,7 @@ constexpr int kCTElems = kCT * kCT;
 struct CholArgs {
     int nt, ntiles, ntasks;
     int n;                       // rows; a row at or past n is an identity row
+    int last;                    // position of the tile row that holds row n - 1
     int solve;                   // 0: factor only, 1: also x = A^{-1} b
     const int *colptr, *rowpos;  // nt + 1, ntiles: per column the positions of its tiles (diagonal first)
     const int *rptr, *rcol, *rslot;   // per row position: the columns left of the diagonal, and the slots

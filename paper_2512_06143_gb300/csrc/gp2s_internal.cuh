@@ -160,7 +160,7 @@ struct gp2s_ctx {
     // and tile structure) with its sizes
     gp2s::DevBuf dense, chol_ints;
     bool chol_plan_valid = false;   // chol_ints belongs to the current pattern
-    int chol_nt = 0, chol_ntiles = 0, chol_ntasks = 0;
+    int chol_nt = 0, chol_ntiles = 0, chol_ntasks = 0, chol_last = 0;
     // adjoint
     gp2s::DevBuf H, gpart;
     // posterior (test points, their bump values / prior variances / outputs, counters, partials)

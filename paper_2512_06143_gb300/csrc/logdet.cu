@@ -453,6 +453,7 @@ extern "C" gp2s_status gp2s_lml_exact_noalloc(int64_t n, const double *X_dev, co
     ca.ntiles = chol_dense_tiles(ca.nt);
     ca.ntasks = ca.ntiles + 2 * ca.nt;
     ca.n = nn;
+    ca.last = ca.nt - 1;
     ca.solve = 1;
     ca.tiles = base;
     ca.dinv = base + kNoAllocVec;
